@@ -17,7 +17,17 @@ namespace as2d {
 constexpr int kMaxBatch = AS2D_MAX_BATCH;
 constexpr int kMaxK = AS2D_MAX_K;
 constexpr int kMaxRows = kMaxBatch * (kMaxK + 1);
-constexpr int kPrefillRows = 64;  // token rows of one prefill pass
+// Token rows of one prefill pass: the smallest of 64, 128 and 256 (one launch
+// of the projections) that holds the call, so that a short instruction keeps
+// a small working state.
+constexpr int kPrefillMaxRows = 256;
+inline int prefill_rows(int n) { return n <= 64 ? 64 : n <= 128 ? 128 : kPrefillMaxRows; }
+
+// What the accept scan does with a request's rows: the verification rule;
+// every row kept and the root taken from the last one (a prefill's last
+// pass); every row kept, root unchanged (its earlier passes, which run no LM
+// head).
+enum AcceptMode : int32_t { kAcceptVerify = 0, kAcceptAll = 1, kAcceptAllNoRoot = 2 };
 
 typedef __nv_bfloat16 bf16;
 
@@ -207,9 +217,9 @@ struct KvState {
   int32_t* cb_dev = nullptr;
   int32_t* cb_host = nullptr;            // pinned, same layout
   int32_t* pf_out = nullptr;             // [2] n_accepted, root of as2d_prefill chunks
-  // as2d_prefill's working state (batch 1, kPrefillRows rows per pass), made
-  // on first use; shares this state's cache, lengths, roots, error flags and
-  // rotary table
+  // as2d_prefill's working state (batch 1, prefill_rows(n) rows per pass), made
+  // on first use and again for a longer call; shares this state's cache,
+  // lengths, roots, error flags and rotary table
   KvState* pf = nullptr;
 };
 
@@ -224,7 +234,7 @@ cudaError_t launch_embed(const RowMap& m, const Model& md, KvState& kv,
                          const int32_t* root_override = nullptr);
 cudaError_t launch_accept(const RowMap& m, const Model& md, KvState& kv,
                           const int32_t* cand, const as2d_verify_out& out,
-                          cudaStream_t st, bool force = false);
+                          cudaStream_t st, AcceptMode mode = kAcceptVerify);
 cudaError_t launch_rollback(KvState& kv, const int32_t* new_len,
                             const int32_t* new_root, cudaStream_t st);
 // Fills kv.rope_full for positions [0, capacity).

@@ -126,11 +126,11 @@ cudaError_t launch_rope_table(const Model& md, KvState& kv, cudaStream_t st) {
 
 cudaError_t launch_accept(const RowMap& m, const Model& md, KvState& kv,
                           const int32_t* cand, const as2d_verify_out& out,
-                          cudaStream_t st, bool force) {
+                          cudaStream_t st, AcceptMode mode) {
   (void)md;
   ++kv.launches;
   AcceptArgs a{m, cand, kv.best, kv.d_len, kv.d_root, kv.d_err + 1, out.n_accepted,
-               out.correction_token, out.greedy, force ? 1 : 0};
+               out.correction_token, out.greedy, mode};
   return launch_pdl(accept_kernel, dim3(m.batch), dim3(32), 0, st, a);
 }
 

@@ -1,6 +1,5 @@
 // small_dev.cuh -- device functions of the embedding gather and the accept
-// scan, shared by the standalone kernels (k_basic.cu) and the persistent
-// verification kernel (k_mk.cu), so both paths compute bit for bit alike.
+// scan (k_basic.cu).
 #pragma once
 
 #include "as2d_internal.h"
@@ -56,7 +55,7 @@ struct AcceptArgs {
   int32_t* n_out;
   int32_t* corr_out;
   int32_t* greedy_out;
-  int32_t force;  // 1: every row is kept whatever the greedy tokens (prefill)
+  int32_t mode;  // AcceptMode
 };
 
 // Accept scan of request b by one warp (App. C.2): g_i from the packed maxima,
@@ -66,9 +65,10 @@ __device__ __forceinline__ void accept_request(const AcceptArgs& a, int b, int l
   const RowMap& m = a.rm;
   const int r0 = m.start[b];
   const int k = m.start[b + 1] - r0 - 1;
-  if (a.force) {
-    // every row kept (prefill, up to kPrefillRows rows): the maxima cleared
-    // 32 rows at a time, the root is the greedy token after the last row
+  if (a.mode != kAcceptVerify) {
+    // every row kept (prefill, up to kPrefillMaxRows rows): the maxima cleared
+    // 32 rows at a time, the root is the greedy token after the last row (in
+    // the pass that runs the LM head)
     int g_last = 0;
     for (int i = lane; i <= k; i += 32) {
       const unsigned long long v = a.best[r0 + i];
@@ -85,9 +85,11 @@ __device__ __forceinline__ void accept_request(const AcceptArgs& a, int b, int l
         a.bad[b] = 0;
       } else {
         a.n_out[b] = k;
-        a.corr_out[b] = g_last;
         a.len[b] += k + 1;
-        a.root[b] = g_last;
+        if (a.mode == kAcceptAll) {
+          a.corr_out[b] = g_last;
+          a.root[b] = g_last;
+        }
       }
     }
     return;

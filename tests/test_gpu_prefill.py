@@ -72,7 +72,7 @@ def test_prefill_matches_oracle(pair):
 @pytest.mark.parametrize("chunks", [[1] * 100, [17, 83], [64, 36], [5, 90, 5], [99, 1]])
 def test_prefill_is_chunking_invariant(pair, chunks):
     """Any split of the suffix into prefill calls gives bitwise the same cache
-    and first token as one call of 100 tokens (passes of 64 + 36 rows):
+    and first token as one call of 100 tokens (one pass):
     pathwise equivalence and batch invariance."""
     cfg = pair.cfg
     instr = [int(t) for t in W.instruction_tokens(cfg, 100, 1)]
@@ -85,6 +85,42 @@ def test_prefill_is_chunking_invariant(pair, chunks):
     assert st.read_state() == ref.read_state()
     st.close()
     ref.close()
+
+
+@pytest.mark.parametrize("n,chunks", [(256, [64, 64, 128]), (257, [64, 193]), (300, [129, 171])])
+def test_prefill_wide_passes(pair, n, chunks):
+    """Passes of up to 256 rows, one row past a pass, and calls that outgrow
+    the working state of the call before them (64 -> 128 -> 256 rows): bitwise
+    the cache and first token of one call."""
+    cfg, cap = pair.cfg, L0 + n + 4
+    instr = torch_tokens(cfg, n)
+
+    def prefill(parts):
+        import torch
+        st = pair.state([L0], cap, [0])
+        first = torch.full((1,), -7, dtype=torch.int32, device="cuda")
+        at = 0
+        for c in parts:
+            st.prefill(instr[at:at + c], first)
+            at += c
+        torch.cuda.synchronize()
+        st.check()
+        return st, int(first.item())
+
+    ref, first_ref = prefill([1] * 3 + [60] * ((n - 3) // 60) + ([(n - 3) % 60] if (n - 3) % 60 else []))
+    for parts in ([n], chunks):
+        st, first = prefill(parts)
+        assert first == first_ref and st.read_state() == ref.read_state() == ([L0 + n], [first])
+        for l in range(cfg.n_layers):
+            for a, b in ((st.kc, ref.kc), (st.vc, ref.vc)):
+                assert np.array_equal(bf16_bits(a[l, 0])[:, :L0 + n], bf16_bits(b[l, 0])[:, :L0 + n])
+        st.close()
+    ref.close()
+
+
+def torch_tokens(cfg, n):
+    import torch
+    return torch.tensor([int(t) for t in W.instruction_tokens(cfg, n, 2)], dtype=torch.int32, device="cuda")
 
 
 def test_prefill_argument_errors(pair):
