@@ -122,20 +122,6 @@ struct AttnArgs {
 
 // ---- finishing the QKV projection from its split-K sums ----------------------
 
-// Projection value of column col (q, k or v head * D + e) for token row gm:
-// the split parts added in rank order, times the row's 1 / rms.
-__device__ __forceinline__ float qkv_value(const AttnArgs& a, int col, int gm) {
-  const float* src = a.qkv_part + ((size_t)(col >> 7) * a.qkv_split * a.qkv_ld + gm) * 128 + (col & 127);
-  float v[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) v[r] = r < a.qkv_split ? src[(size_t)r * a.qkv_ld * 128] : 0.f;
-  float acc = 0.f;
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-    if (r < a.qkv_split) acc += v[r];
-  return acc * a.qkv_rinv[gm];
-}
-
 // Byte offset of element (row r, column e) in a 128-row operand image of
 // 128-byte-swizzled K-major bf16: 64-column regions of kRegion bytes, 16-byte
 // chunk j of row r stored at chunk j ^ (r mod 8).
@@ -145,50 +131,111 @@ __device__ __forceinline__ uint32_t img_off(int r, int e) {
          (uint32_t)((e & 7) << 1);
 }
 
-// One CTA of D / 2 threads per (token row, head); thread e forms the pair
-// (e, e + D/2).  Rotate-half RoPE: x' = x cos - x_p sin at e, x_p cos + x sin
-// at e + D/2.
+// One warp per (token row, head); lane l forms the pairs (e, e + D/2) of e =
+// V l .. V l + V - 1.  Rotate-half RoPE: x' = x cos - x_p sin at e, x_p cos +
+// x sin at e + D/2.  Bound by latency, as the residual projections' finishing
+// kernel is (whose comment has the figures of both): addresses before the
+// wait, every load issued before any is used, a warp to a row of a head.  The
+// dependent launch is triggered after the wait: attention CTAs that start
+// before it read the requests' lengths (and measured slower: 7B k = 8 2784 ->
+// 2810 us).
+constexpr int kQkvWarps = 8;  // heads (warps) of one CTA
 template <int D>
-__global__ void __launch_bounds__(D / 2) qkv_finish_kernel(AttnArgs a) {
+__global__ void __launch_bounds__(32 * kQkvWarps) qkv_finish_kernel(const __grid_constant__ AttnArgs a) {
+  constexpr int H2 = D / 2, V = H2 / 32;
+  const int gm = blockIdx.x, head = blockIdx.y * kQkvWarps + threadIdx.y, e = V * threadIdx.x;
+  const int b = row_request(a.rm, gm), r0 = a.rm.start[b], i = gm - r0, rows = a.rm.start[b + 1] - r0;
+  const bool live = head < a.nq + 2 * a.nkv;
+  const bool is_q = head < a.nq, rotate = head < a.nq + a.nkv;
+  // the split parts of columns head D + e .. and head D + e + H2 ..
+  const int c0 = head * D + e, c1 = c0 + H2;
+  const size_t part = (size_t)a.qkv_ld * 128;
+  const float* s0 = a.qkv_part + ((size_t)(c0 >> 7) * a.qkv_split * a.qkv_ld + gm) * 128 + (c0 & 127);
+  const float* s1 = a.qkv_part + ((size_t)(c1 >> 7) * a.qkv_split * a.qkv_ld + gm) * 128 + (c1 & 127);
+  const float2* csp = a.rope + (size_t)gm * H2 + e;
+  // where the results go: the query image's rows 2q (hi) and 2q + 1 (lo), or
+  // the cache entry at the request's length + i
+  const int G = a.nq / a.nkv;
+  const int g = is_q ? head / G : (rotate ? head - a.nq : head - a.nq - a.nkv);
+  const int qg = i * G + (head - g * G), qt = qg / kQT, q = qg - qt * kQT;
+  uint8_t* img = a.qimg + ((size_t)(b * a.nkv + g) * a.qt_max + qt) * (size_t)(256 * D);
+  bf16* dst = (rotate ? a.kc : a.vc) + (((size_t)a.layer * a.batch + b) * a.nkv + g) * a.cap * D + e;
   ptx::griddep_wait();
   ptx::griddep_launch_dependents();
-  constexpr int H2 = D / 2;
-  const int gm = blockIdx.x, head = blockIdx.y, e = threadIdx.x;
-  const int b = row_request(a.rm, gm), i = gm - a.rm.start[b];
-  // every load is issued before any is used: one memory round trip
+  if (!live) return;
   const int len_b = a.len[b];
-  const float x = qkv_value(a, head * D + e, gm), xp = qkv_value(a, head * D + e + H2, gm);
-  const bool rotate = head < a.nq + a.nkv;
-  const float2 cs = rotate ? a.rope[(size_t)gm * H2 + e] : make_float2(1.f, 0.f);
-  if (!rows_fit(len_b, a.rm.start[b + 1] - a.rm.start[b], a.cap)) return;  // flagged
-  const int pos = len_b + i;
-  float y0, y1;
-  if (rotate) {
-    y0 = fmaf(x, cs.x, -(xp * cs.y));
-    y1 = fmaf(xp, cs.x, x * cs.y);
-  } else {
-    y0 = x;
-    y1 = xp;
+  const float rinv = a.qkv_rinv[gm];
+  float x[V], xp[V];
+  float2 cs[V];
+  {
+    float v0[8][V], v1[8][V];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (r < a.qkv_split) {
+        if constexpr (V == 2) {
+          const float2 t0 = __ldcg(reinterpret_cast<const float2*>(s0 + r * part));
+          const float2 t1 = __ldcg(reinterpret_cast<const float2*>(s1 + r * part));
+          v0[r][0] = t0.x, v0[r][1] = t0.y;
+          v1[r][0] = t1.x, v1[r][1] = t1.y;
+        } else {
+          v0[r][0] = __ldcg(s0 + r * part);
+          v1[r][0] = __ldcg(s1 + r * part);
+        }
+      }
+#pragma unroll
+    for (int u = 0; u < V; ++u) cs[u] = rotate ? csp[u] : make_float2(1.f, 0.f);
+    // the parts in rank order, times the row's 1 / rms
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < a.qkv_split) {
+          t0 += v0[r][u];
+          t1 += v1[r][u];
+        }
+      x[u] = t0 * rinv;
+      xp[u] = t1 * rinv;
+    }
   }
-  if (head < a.nq) {
-    const int G = a.nq / a.nkv, g = head / G;
-    const int qg = i * G + (head - g * G);
-    const int qt = qg / kQT, q = qg - qt * kQT;
-    uint8_t* img = a.qimg + ((size_t)(b * a.nkv + g) * a.qt_max + qt) * (size_t)(256 * D);
-    const float v0 = y0 * a.qscale, v1 = y1 * a.qscale;
-    const bf16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
-    *reinterpret_cast<bf16*>(img + img_off(2 * q, e)) = h0;
-    *reinterpret_cast<bf16*>(img + img_off(2 * q, e + H2)) = h1;
-    *reinterpret_cast<bf16*>(img + img_off(2 * q + 1, e)) =
-        __float2bfloat16_rn(v0 - __bfloat162float(h0));
-    *reinterpret_cast<bf16*>(img + img_off(2 * q + 1, e + H2)) =
-        __float2bfloat16_rn(v1 - __bfloat162float(h1));
+  if (!rows_fit(len_b, rows, a.cap)) return;  // flagged
+  float y0[V], y1[V];
+#pragma unroll
+  for (int u = 0; u < V; ++u) {
+    y0[u] = rotate ? fmaf(x[u], cs[u].x, -(xp[u] * cs[u].y)) : x[u];
+    y1[u] = rotate ? fmaf(xp[u], cs[u].x, x[u] * cs[u].y) : xp[u];
+  }
+  // V consecutive bf16 (4-byte aligned for V = 2)
+  auto put = [](void* to, const bf16* v) {
+    if constexpr (V == 2)
+      *reinterpret_cast<__nv_bfloat162*>(to) = __halves2bfloat162(v[0], v[1]);
+    else
+      *reinterpret_cast<bf16*>(to) = v[0];
+  };
+  if (is_q) {
+    bf16 h0[V], h1[V], l0[V], l1[V];
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const float w0 = y0[u] * a.qscale, w1 = y1[u] * a.qscale;
+      h0[u] = __float2bfloat16_rn(w0);
+      h1[u] = __float2bfloat16_rn(w1);
+      l0[u] = __float2bfloat16_rn(w0 - __bfloat162float(h0[u]));
+      l1[u] = __float2bfloat16_rn(w1 - __bfloat162float(h1[u]));
+    }
+    put(img + img_off(2 * q, e), h0);
+    put(img + img_off(2 * q, e + H2), h1);
+    put(img + img_off(2 * q + 1, e), l0);
+    put(img + img_off(2 * q + 1, e + H2), l1);
   } else {
-    const bool is_k = head < a.nq + a.nkv;
-    const int g = is_k ? head - a.nq : head - a.nq - a.nkv;
-    bf16* dst = (is_k ? a.kc : a.vc) + ((((size_t)a.layer * a.batch + b) * a.nkv + g) * a.cap + pos) * D;
-    dst[e] = __float2bfloat16_rn(y0);
-    dst[e + H2] = __float2bfloat16_rn(y1);
+    bf16 k0[V], k1[V];
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      k0[u] = __float2bfloat16_rn(y0[u]);
+      k1[u] = __float2bfloat16_rn(y1[u]);
+    }
+    dst += (size_t)(len_b + i) * D;
+    put(dst, k0);
+    put(dst + H2, k1);
   }
 }
 
@@ -1327,18 +1374,19 @@ cudaError_t launch_attention_split(const RowMap& m, const Model& md, KvState& kv
     a.cl_start[b + 1] = a.cl_start[b] + attn_q_tiles(m.start[b + 1] - m.start[b], G) *
                                             ((a.n_ch[b] + halves - 1) / halves);
   const int clusters = a.cl_start[kv.batch];
-  const dim3 gf(m.rows, c.n_q_heads + 2 * c.n_kv_heads);
+  const dim3 gf(m.rows, (c.n_q_heads + 2 * c.n_kv_heads + kQkvWarps - 1) / kQkvWarps);
+  const dim3 bf(32, kQkvWarps);
   cudaError_t e;
   kv.launches += 2;
   if (c.head_dim == 128) {
-    e = launch_pdl(qkv_finish_kernel<128>, gf, dim3(64), 0, st, a);
+    e = launch_pdl(qkv_finish_kernel<128>, gf, bf, 0, st, a);
     if (e == cudaSuccess)
       e = quad     ? launch_attn4<128>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : narrow ? launch_attn<128, true, false>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : pair ? launch_attn<128, false, true>(kv.tm_kc, kv.tm_vc, a, clusters, st)
                  : launch_attn<128, false, false>(kv.tm_kc, kv.tm_vc, a, clusters, st);
   } else {
-    e = launch_pdl(qkv_finish_kernel<64>, gf, dim3(32), 0, st, a);
+    e = launch_pdl(qkv_finish_kernel<64>, gf, bf, 0, st, a);
     if (e == cudaSuccess)
       e = quad     ? launch_attn4<64>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : narrow ? launch_attn<64, true, false>(kv.tm_kc, kv.tm_vc, a, clusters, st)

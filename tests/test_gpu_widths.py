@@ -1,0 +1,54 @@
+"""Calls of every token-row padding on a decoder whose projections end in odd
+and partial tiles (hidden 384: 3 tiles of 128; gate/up 7; vocabulary 8 and a
+fraction; 10 heads): the first request of each call against the oracle, and
+every request's rows against the same request verified alone, bit for bit."""
+import numpy as np
+import pytest
+
+from synth import workloads as W
+from tests.helpers import LOGIT_TOL, Pair, run_gpu_block
+
+pytestmark = pytest.mark.gpu
+
+ODD = W.ModelConfig("odd", 2, 384, 6, 2, 64, 448, 1032)
+CAP = 256
+
+
+@pytest.fixture(scope="module")
+def pair():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    return Pair(ODD, seed=0, gains="random")
+
+
+# requests x rows: 1, 15, 16, 17 (a finishing CTA's rows), then one call past
+# each padding's lower edge and at 256, 257 and 272 rows (two launches)
+@pytest.mark.parametrize("rows", [[1], [15], [16], [17], [17, 16], [17, 17, 15], [16] * 4, [17] * 4, [17] * 6,
+                                  [17] * 8, [17] * 10, [17] * 12, [16] * 16, [17] * 15 + [2], [17] * 16],
+                         ids=lambda r: f"{sum(r)}rows")
+def test_rows(pair, rows):
+    cfg, n = pair.cfg, len(rows)
+    rng = np.random.default_rng(sum(rows))
+    lens = [int(x) for x in rng.integers(1, CAP - 20, size=n)]
+    roots = [int(x) for x in rng.integers(0, cfg.vocab, size=n)]
+    cands = [[int(t) for t in rng.integers(0, cfg.vocab, size=r - 1)] for r in rows]
+    st = pair.state(lens, CAP, roots)
+    acc, corr, greedy, logits = run_gpu_block(st, cfg, cands)
+    st.check()
+    kc, vc = st.kc.clone(), st.vc.clone()
+    st.close()
+    oc = pair.oracle_cache(lens[0], CAP)
+    want = pair.oracle.verify_block(oc, lens[0], roots[0], cands[0])
+    assert np.max(np.abs(want["logits"] - logits[:rows[0]])) <= LOGIT_TOL
+    at = 0
+    for b in range(n):
+        one = pair.state([lens[b]], CAP, [roots[b]])
+        # the request's own prefix (positions below its length)
+        one.kc[:, 0, :, :lens[b]] = kc[:, b, :, :lens[b]]
+        one.vc[:, 0, :, :lens[b]] = vc[:, b, :, :lens[b]]
+        a1, c1, g1, l1 = run_gpu_block(one, cfg, [cands[b]])
+        assert np.array_equal(l1, logits[at:at + rows[b]]), f"request {b}"
+        assert a1[0] == acc[b] and c1[0] == corr[b] and np.array_equal(g1, greedy[at:at + rows[b]])
+        one.close()
+        at += rows[b]
