@@ -63,7 +63,8 @@ EncodeTiledFn encode_fn() {
 // Row-major bf16 matrix [outer][inner] viewed by TMA in boxes of
 // box_inner x box_outer elements with 128-byte swizzling.
 bool encode_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer,
-               uint32_t box_inner, uint32_t box_outer) {
+               uint32_t box_inner, uint32_t box_outer,
+               CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {inner, outer};
@@ -71,8 +72,27 @@ bool encode_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t oute
   cuuint32_t box[2] = {box_inner, box_outer};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// A packed weight matrix (k_pack.cu), one 128 x 64 unit to a box, copied as it
+// lies (it is stored in its shared-memory image).
+bool encode_packed(CUtensorMap* map, const bf16* base, size_t elems) {
+  return encode_2d(map, base, 64, elems / 64, 64, 128, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
+// The activation operand [rows][K] for every token-row padding up to nb_max:
+// boxes of nb rows, and those of a pair of CTAs (nb rows up to 128, nb / 2 above).
+bool encode_operand(CUtensorMap* maps, CUtensorMap* pair, const bf16* base, int K, uint64_t rows,
+                    int nb_max) {
+  for (int i = 0; i < kNbCount && kNbSet[i] <= nb_max; ++i) {
+    const int nb = kNbSet[i];
+    if (!encode_2d(&maps[i], base, K, rows, 64, nb) ||
+        !encode_2d(&pair[i], base, K, rows, 64, nb <= 128 ? nb : nb / 2))
+      return false;
+  }
+  return true;
 }
 
 }  // namespace
@@ -189,6 +209,11 @@ extern "C" as2d_status as2d_model_load(const as2d_config* cfg,
     LOAD_TRY(pack_weights(lm, (int)V, (int)H, segs, rows, 1, false, 0));
   }
   LOAD_TRY(launch_f32_from_bf16(fnorm, w->final_norm, H, 0));
+  bool maps = encode_packed(&m.tm_lm_head, lm, lm_packed);
+  m.tm_qkv.resize(L);
+  m.tm_o.resize(L);
+  m.tm_gu.resize(L);
+  m.tm_down.resize(L);
   m.embed = embed;
   m.lm_head = lm;
   m.final_norm = fnorm;
@@ -221,6 +246,9 @@ extern "C" as2d_status as2d_model_load(const as2d_config* cfg,
     }
     LOAD_TRY(launch_f32_from_bf16(an, w->attn_norm[l], H, 0));
     LOAD_TRY(launch_f32_from_bf16(mn, w->mlp_norm[l], H, 0));
+    maps = maps && encode_packed(&m.tm_qkv[l], qkv, qkv_packed) &&
+           encode_packed(&m.tm_o[l], wo, o_packed) && encode_packed(&m.tm_gu[l], gu, gu_packed) &&
+           encode_packed(&m.tm_down[l], wd, down_packed);
     m.w_qkv.push_back(qkv);
     m.w_o.push_back(wo);
     m.w_gu.push_back(gu);
@@ -229,6 +257,7 @@ extern "C" as2d_status as2d_model_load(const as2d_config* cfg,
     m.mlp_norm.push_back(mn);
   }
   LOAD_TRY(cudaDeviceSynchronize());
+  if (!maps) return fail_free("cuTensorMapEncodeTiled failed for a weight matrix");
 #undef LOAD_TRY
   *out = mh;
   return AS2D_OK;
@@ -261,12 +290,13 @@ as2d_status alloc_work(KvState& s, const Model& m, int batch, int capacity,
   s.nb_max = nb_for_rows(s.max_rows);
   s.rows_alloc = s.max_rows > s.nb_max ? s.max_rows : s.nb_max;
   const size_t R = s.rows_alloc, H = m.cfg.hidden, F = m.cfg.ffn;
+  const size_t ws_ctas = m.sm_count > 2 ? m.sm_count : 2;  // a projection's grid is even
   const size_t max_tiles = ((size_t)(m.cfg.vocab > 2 * F ? m.cfg.vocab : 2 * F) + 127) / 128 + 64;
   size_t bytes = 4096 + 3 * align_up((size_t)(batch + 1) * 4, 256);
   bytes += align_up(R * H * 4, 256) + align_up(2 * R * H * 2, 256) +
            align_up(2 * R * m.q_dim * 2, 256) + align_up(2 * R * F * 2, 256) + align_up(R * 8, 256) +
            align_up(R * (m.cfg.head_dim / 2) * 8, 256) + align_up(R * (H / 128) * 4, 256) +
-           align_up((size_t)m.sm_count * 2 * s.nb_max * 128 * 4, 256) + align_up(max_tiles * 4, 256);
+           align_up(ws_ctas * 2 * s.nb_max * 128 * 4, 256) + align_up(max_tiles * 4, 256);
   s.qkv_split = qkv_split_for(m);
   const size_t qkv_tiles = (size_t)(m.qkv_rows + 127) / 128;
   bytes += align_up(qkv_tiles * s.qkv_split * R * 128 * 4, 256) + align_up(R * 4, 256);
@@ -295,7 +325,7 @@ as2d_status alloc_work(KvState& s, const Model& m, int batch, int capacity,
   s.best = cv.take<unsigned long long>(R);
   s.rope = cv.take<float2>(R * (m.cfg.head_dim / 2));
   s.ss = cv.take<float>(R * (H / 128));
-  s.ws = cv.take<float>((size_t)m.sm_count * 2 * s.nb_max * 128);
+  s.ws = cv.take<float>(ws_ctas * 2 * s.nb_max * 128);
   s.ws_sms = m.sm_count;
   s.counters = cv.take<int>(max_tiles);
   s.n_counters = (int)max_tiles;
@@ -310,13 +340,9 @@ as2d_status alloc_work(KvState& s, const Model& m, int batch, int capacity,
                              (int64_t)m.cfg.n_layers * batch * m.cfg.n_kv_heads) &&
             encode_cache_map(&s.tm_vc, s.v_cache, m.cfg.head_dim, capacity,
                              (int64_t)m.cfg.n_layers * batch * m.cfg.n_kv_heads);
-  for (int i = 0; i < kNbCount && ok; ++i) {
-    const int nb = kNbSet[i];
-    if (nb > s.nb_max) break;
-    ok = encode_2d(&s.tm_xn[i], s.xn, H, 2 * R, 64, nb) &&
-         encode_2d(&s.tm_ao[i], s.ao, m.q_dim, 2 * R, 64, nb) &&
-         encode_2d(&s.tm_u[i], s.u, F, 2 * R, 64, nb);
-  }
+  ok = ok && encode_operand(s.tm_xn, s.tm_xn_pair, s.xn, (int)H, 2 * R, s.nb_max) &&
+       encode_operand(s.tm_ao, s.tm_ao_pair, s.ao, m.q_dim, 2 * R, s.nb_max) &&
+       encode_operand(s.tm_u, s.tm_u_pair, s.u, (int)F, 2 * R, s.nb_max);
   if (!ok) {
     cudaFree(s.work);
     s.work = nullptr;
@@ -446,17 +472,21 @@ int as2d::qkv_split_for(const Model& m) {
 
 namespace {
 
+// The activation operand of a projection.
+struct Operand {
+  const CUtensorMap *maps, *pair;  // per token-row padding
+};
+
 cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, const bf16* w,
-                       const CUtensorMap* xmaps, int N, int K, TcParams p, cudaStream_t st,
-                       int first_row = 0) {
+                       const CUtensorMap& wmap, const Operand& x, int N, int K, TcParams p,
+                       cudaStream_t st, int first_row = 0) {
   p.w = w;
   p.N = N;
   p.K = K;
   p.n_tiles = (N + 127) / 128;
   p.kb = (K + 63) / 64;
-  p.units = (long long)p.n_tiles * p.kb;
-  // Work split (all of it a function of N, K and the device only, so a
-  // row's sums are added in the same order whatever the number of rows):
+  // Work split (tc_range; all of it a function of N, K and the device only, so
+  // a row's sums are added in the same order whatever the number of rows):
   //   QKV (TC_PART): K split evenly over qkv_split CTAs per tile, sums
   //     finished by qkv_finish_kernel;
   //   at least 90% as many tiles as SMs (gate/up): whole tiles per CTA,
@@ -467,23 +497,29 @@ cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, co
   //     held by the attention start late); residual projections leave their
   //     split tiles to tc_resid_finish_kernel, the LM head finishes them in
   //     the GEMM (last CTA of a tile).
-  p.grid = (int)(p.units < m.sm_count ? p.units : m.sm_count);
-  if (epi == TC_RESID && p.units / 4 < p.grid) p.grid = p.units >= 4 ? (int)(p.units / 4) : 1;
+  const int pairs = (p.n_tiles + 1) / 2, units = pairs * p.kb;
+  const int most = m.sm_count > 2 ? m.sm_count / 2 : 1;  // groups that the SMs hold
+  int work = units;
   p.split = 0;
   p.defer = epi == TC_RESID ? 1 : 0;
+  p.groups = units < most ? units : most;
+  if (epi == TC_RESID && units / 4 < p.groups) p.groups = units >= 4 ? units / 4 : 1;
   if (epi == TC_SWIGLU && p.n_tiles * 10 >= m.sm_count * 9) {
-    const int per = (p.n_tiles + m.sm_count - 1) / m.sm_count;
+    const int per = (pairs + most - 1) / most;
     p.split = 1;
-    p.grid = (p.n_tiles + per - 1) / per;
-    p.defer = 0;
+    p.groups = (pairs + per - 1) / per;
+    work = pairs;
   }
   if (epi == TC_PART) {
     p.split = s.qkv_split;
-    p.grid = p.n_tiles * p.split;
+    p.groups = pairs * p.split;
+    work = pairs;
     p.part = s.qkv_part;
     p.part_rinv = s.qkv_rinv;
     p.part_ld = s.rows_alloc;
   }
+  p.gq = work / p.groups;
+  p.gr = work % p.groups;
   p.ws = s.ws;
   p.counters = s.counters;
   p.err = s.d_err;
@@ -492,17 +528,17 @@ cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, co
   for (int row0 = first_row; row0 < rm.rows; row0 += 256) {
     p.row0 = row0;
     p.rows = rm.rows - row0 < 256 ? rm.rows - row0 : 256;
-    const int nb = nb_for_rows(p.rows);
-    const CUtensorMap& x = xmaps[nb_index(nb)];
+    const int nb = nb_for_rows(p.rows), i = nb_index(nb);
+    const TcMaps maps{&x.maps[i], &x.pair[i], &wmap};
     cudaError_t e;
     switch (epi) {
-      case TC_PART: e = tc_gemm_part(nb, x, p, st); break;
-      case TC_RESID: e = tc_gemm_resid(nb, x, p, st); break;
-      case TC_SWIGLU: e = tc_gemm_swiglu(nb, x, p, st); break;
-      default: e = tc_gemm_logits(nb, x, p, st); break;
+      case TC_PART: e = tc_gemm_part(nb, maps, p, st); break;
+      case TC_RESID: e = tc_gemm_resid(nb, maps, p, st); break;
+      case TC_SWIGLU: e = tc_gemm_swiglu(nb, maps, p, st); break;
+      default: e = tc_gemm_logits(nb, maps, p, st); break;
     }
     if (e != cudaSuccess) return e;
-    s.launches += (p.defer && p.grid >= 2) ? 2 : 1;
+    s.launches += (p.defer && p.groups >= 2) ? 2 : 1;
   }
   return cudaSuccess;
 }
@@ -554,18 +590,19 @@ as2d_status run_block(KvState& s, const int32_t* cand, const int32_t* k,
   tp.eps = c.rms_eps;
   tp.hidden = c.hidden;
   const int H = c.hidden, F = c.ffn;
+  const Operand xn{s.tm_xn, s.tm_xn_pair}, ao{s.tm_ao, s.tm_ao_pair}, u{s.tm_u, s.tm_u_pair};
   for (int l = 0; l < c.n_layers; ++l) {
-    LAUNCH(AS2D_KERNEL_QKV, tc_project(TC_PART, m, s, rm, m.w_qkv[l], s.tm_xn, m.qkv_rows, H, tp, st));
+    LAUNCH(AS2D_KERNEL_QKV, tc_project(TC_PART, m, s, rm, m.w_qkv[l], m.tm_qkv[l], xn, m.qkv_rows, H, tp, st));
     LAUNCH(AS2D_KERNEL_ATTENTION, launch_attention_split(rm, m, s, l, st));
     tp.g_next = m.mlp_norm[l];
-    LAUNCH(AS2D_KERNEL_O, tc_project(TC_RESID, m, s, rm, m.w_o[l], s.tm_ao, H, m.q_dim, tp, st));
-    LAUNCH(AS2D_KERNEL_GATE_UP, tc_project(TC_SWIGLU, m, s, rm, m.w_gu[l], s.tm_xn, 2 * F, H, tp, st));
+    LAUNCH(AS2D_KERNEL_O, tc_project(TC_RESID, m, s, rm, m.w_o[l], m.tm_o[l], ao, H, m.q_dim, tp, st));
+    LAUNCH(AS2D_KERNEL_GATE_UP, tc_project(TC_SWIGLU, m, s, rm, m.w_gu[l], m.tm_gu[l], xn, 2 * F, H, tp, st));
     tp.g_next = (l + 1 < c.n_layers) ? m.attn_norm[l + 1] : m.final_norm;
-    LAUNCH(AS2D_KERNEL_DOWN, tc_project(TC_RESID, m, s, rm, m.w_down[l], s.tm_u, H, F, tp, st));
+    LAUNCH(AS2D_KERNEL_DOWN, tc_project(TC_RESID, m, s, rm, m.w_down[l], m.tm_down[l], u, H, F, tp, st));
   }
   // a prefill needs one token, the greedy one after its last row
   if (mode != kAcceptAllNoRoot)
-    LAUNCH(AS2D_KERNEL_LM_HEAD, tc_project(TC_LOGITS, m, s, rm, m.lm_head, s.tm_xn, c.vocab, H, tp,
+    LAUNCH(AS2D_KERNEL_LM_HEAD, tc_project(TC_LOGITS, m, s, rm, m.lm_head, m.tm_lm_head, xn, c.vocab, H, tp,
                                            st, mode == kAcceptAll ? rm.rows - 1 : 0));
   LAUNCH(AS2D_KERNEL_OTHER, launch_accept(rm, m, s, cand, *out, st, mode));
   for (int b = 0; b < s.batch; ++b) s.len_upper[b] += (k ? k[b] : 0) + 1;
@@ -947,6 +984,7 @@ extern "C" as2d_status as2d_decode_step_static(as2d_model* mh, void* k_cache, vo
   rm.start[1] = 1;
   as2d_verify_out out{(int32_t*)(b + kOffErr + 16), correction_token, nullptr, logits};
   const int H = c.hidden, F = c.ffn;
+  const Operand xn{s.tm_xn, s.tm_xn_pair}, ao{s.tm_ao, s.tm_ao_pair}, u{s.tm_u, s.tm_u_pair};
   LAUNCH(AS2D_KERNEL_OTHER, launch_embed(rm, m, s, nullptr, st));
   TcParams tp{};
   tp.h = s.h;
@@ -961,15 +999,15 @@ extern "C" as2d_status as2d_decode_step_static(as2d_model* mh, void* k_cache, vo
   tp.eps = c.rms_eps;
   tp.hidden = c.hidden;
   for (int l = 0; l < c.n_layers; ++l) {
-    LAUNCH(AS2D_KERNEL_QKV, tc_project(TC_PART, m, s, rm, m.w_qkv[l], s.tm_xn, m.qkv_rows, H, tp, st));
+    LAUNCH(AS2D_KERNEL_QKV, tc_project(TC_PART, m, s, rm, m.w_qkv[l], m.tm_qkv[l], xn, m.qkv_rows, H, tp, st));
     LAUNCH(AS2D_KERNEL_ATTENTION, launch_attention_split(rm, m, s, l, st));
     tp.g_next = m.mlp_norm[l];
-    LAUNCH(AS2D_KERNEL_O, tc_project(TC_RESID, m, s, rm, m.w_o[l], s.tm_ao, H, m.q_dim, tp, st));
-    LAUNCH(AS2D_KERNEL_GATE_UP, tc_project(TC_SWIGLU, m, s, rm, m.w_gu[l], s.tm_xn, 2 * F, H, tp, st));
+    LAUNCH(AS2D_KERNEL_O, tc_project(TC_RESID, m, s, rm, m.w_o[l], m.tm_o[l], ao, H, m.q_dim, tp, st));
+    LAUNCH(AS2D_KERNEL_GATE_UP, tc_project(TC_SWIGLU, m, s, rm, m.w_gu[l], m.tm_gu[l], xn, 2 * F, H, tp, st));
     tp.g_next = (l + 1 < c.n_layers) ? m.attn_norm[l + 1] : m.final_norm;
-    LAUNCH(AS2D_KERNEL_DOWN, tc_project(TC_RESID, m, s, rm, m.w_down[l], s.tm_u, H, F, tp, st));
+    LAUNCH(AS2D_KERNEL_DOWN, tc_project(TC_RESID, m, s, rm, m.w_down[l], m.tm_down[l], u, H, F, tp, st));
   }
-  LAUNCH(AS2D_KERNEL_LM_HEAD, tc_project(TC_LOGITS, m, s, rm, m.lm_head, s.tm_xn, c.vocab, H, tp, st));
+  LAUNCH(AS2D_KERNEL_LM_HEAD, tc_project(TC_LOGITS, m, s, rm, m.lm_head, m.tm_lm_head, xn, c.vocab, H, tp, st));
   LAUNCH(AS2D_KERNEL_OTHER, launch_accept(rm, m, s, nullptr, out, st));
   // the call's device error bits, for the caller (a copy, not an allocation)
   if (error_bits)

@@ -72,16 +72,16 @@ struct TcParams {
   int lo_row;            // operand buffers hold hi rows [0, R), lo rows [R, 2R): R
   int N, K;              // logical W is [N][K]
   int n_tiles, kb;       // 128-row tiles, 64-column k-blocks
-  long long units;       // n_tiles * kb
-  int grid;              // CTAs
-  int split;             // TC_PART: CTAs per tile (K split), else 0 (stream-K)
+  int groups;            // CTA pairs: the grid is 2 groups (tc_range)
+  int gq, gr;            // work of a group: gq units (split 1: tile pairs), one more for the first gr
+  int split;             // 0: stream-K; 1: whole tiles; TC_PART: CTAs per tile (K split)
   int defer;             // stream-K: split tiles are finished by tc_resid_finish_kernel
   float* part;           // TC_PART: [tile][split][part_ld][128] fp32 sums
   float* part_rinv;      // TC_PART: [part_ld] 1 / rms of each token row
   int part_ld;           // rows_alloc
   int rows;              // token rows handled by this launch
   int row0;              // first token row of this launch
-  float* ws;             // [grid][2][NB][128] partial tiles
+  float* ws;             // [2 groups][2][NB][128] partial tiles
   int* counters;         // [n_tiles] arrivals; zero between launches
   int* err;
   unsigned long long timeout_ns;
@@ -107,21 +107,32 @@ struct TcParams {
 // while its predecessor in the stream is still running; every kernel of the
 // library calls griddepcontrol.wait before it touches memory that an earlier
 // kernel of the stream wrote.
+// cluster: CTAs per thread-block cluster (along x).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t st, Args... args) {
+                       cudaStream_t st, int cluster, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
+
+// TMA descriptors of one projection launch: the activation operand for one
+// CTA per tile and for a pair of CTAs per two tiles, and the weights.
+struct TcMaps {
+  const CUtensorMap *x, *x_pair, *w;
+};
 
 struct Model {
   as2d_config cfg;
@@ -138,8 +149,11 @@ struct Model {
   // projection weights, packed tile-major (k_pack.cu)
   std::vector<const bf16*> w_qkv;   // logical [(nq + 2 nkv) d][H]: q rows, k rows, v rows
   std::vector<const bf16*> w_o;     // logical [H][nq d]
-  std::vector<const bf16*> w_gu;    // logical [2F][H]: per 128 rows, 64 gate then 64 up
+  std::vector<const bf16*> w_gu;    // logical [2F][H]: per 32 rows, 16 gate then 16 up
   std::vector<const bf16*> w_down;  // logical [H][F]
+  // the packed weights as [units * 128][64] bf16, a unit to a box
+  CUtensorMap tm_lm_head;
+  std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
   std::vector<const float*> attn_norm, mlp_norm;  // fp32 gains [H]
 };
 
@@ -201,8 +215,10 @@ struct KvState {
   float2* attn_ml = nullptr; // [batch][n_kv][qt][chunks][64] (max, sum) base 2
   int* attn_cnt = nullptr;   // [batch][n_kv][qt][8] chunks arrived per 8-row group; zero between launches
   int n_attn_cnt = 0;
-  // TMA descriptors of the activation operands, per token-row padding
+  // TMA descriptors of the activation operands, per token-row padding, and
+  // the ones that a pair of CTAs loads through (half boxes above 128 rows)
   CUtensorMap tm_xn[kNbCount], tm_ao[kNbCount], tm_u[kNbCount];
+  CUtensorMap tm_xn_pair[kNbCount], tm_ao_pair[kNbCount], tm_u_pair[kNbCount];
   // TMA descriptors of the caches: [n_layers * batch * n_kv][capacity][d]
   CUtensorMap tm_kc, tm_vc;
   // limit of the kernels' pipeline waits (as2d_kv_set_wait_limit)
@@ -258,13 +274,10 @@ cudaError_t launch_attention_split(const RowMap& m, const Model& md, KvState& kv
 
 // Tensor-core GEMM launchers (k_tc_*.cu), one per fused epilogue.
 int qkv_split_for(const Model& m);
-cudaError_t tc_gemm_part(int nb, const CUtensorMap& x, const TcParams& p, cudaStream_t st);
-cudaError_t tc_gemm_resid(int nb, const CUtensorMap& x, const TcParams& p,
-                          cudaStream_t st);
-cudaError_t tc_gemm_swiglu(int nb, const CUtensorMap& x, const TcParams& p,
-                           cudaStream_t st);
-cudaError_t tc_gemm_logits(int nb, const CUtensorMap& x, const TcParams& p,
-                           cudaStream_t st);
+cudaError_t tc_gemm_part(int nb, const TcMaps& x, const TcParams& p, cudaStream_t st);
+cudaError_t tc_gemm_resid(int nb, const TcMaps& x, const TcParams& p, cudaStream_t st);
+cudaError_t tc_gemm_swiglu(int nb, const TcMaps& x, const TcParams& p, cudaStream_t st);
+cudaError_t tc_gemm_logits(int nb, const TcMaps& x, const TcParams& p, cudaStream_t st);
 
 cudaError_t launch_f32_from_bf16(float* dst, const void* src, int64_t n,
                                  cudaStream_t st);

@@ -1379,14 +1379,14 @@ cudaError_t launch_attention_split(const RowMap& m, const Model& md, KvState& kv
   cudaError_t e;
   kv.launches += 2;
   if (c.head_dim == 128) {
-    e = launch_pdl(qkv_finish_kernel<128>, gf, bf, 0, st, a);
+    e = launch_pdl(qkv_finish_kernel<128>, gf, bf, 0, st, 1, a);
     if (e == cudaSuccess)
       e = quad     ? launch_attn4<128>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : narrow ? launch_attn<128, true, false>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : pair ? launch_attn<128, false, true>(kv.tm_kc, kv.tm_vc, a, clusters, st)
                  : launch_attn<128, false, false>(kv.tm_kc, kv.tm_vc, a, clusters, st);
   } else {
-    e = launch_pdl(qkv_finish_kernel<64>, gf, bf, 0, st, a);
+    e = launch_pdl(qkv_finish_kernel<64>, gf, bf, 0, st, 1, a);
     if (e == cudaSuccess)
       e = quad     ? launch_attn4<64>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : narrow ? launch_attn<64, true, false>(kv.tm_kc, kv.tm_vc, a, clusters, st)

@@ -111,7 +111,7 @@ __global__ void f32_from_bf16_kernel(float* dst, const bf16* src, int64_t n) {
 cudaError_t launch_embed(const RowMap& m, const Model& md, KvState& kv,
                          const int32_t* cand, cudaStream_t st, const int32_t* root_override) {
   ++kv.launches;
-  return launch_pdl(embed_kernel, dim3(m.rows), dim3(128), 0, st, m, cand,
+  return launch_pdl(embed_kernel, dim3(m.rows), dim3(128), 0, st, 1, m, cand,
                     (const int32_t*)kv.d_root, root_override, (const bf16*)md.embed, md.cfg.hidden,
                     md.cfg.vocab, kv.h, kv.d_err, kv.d_err + 1, (const int32_t*)kv.d_len,
                     kv.capacity, kv.rope, (const float2*)kv.rope_full, md.cfg.head_dim,
@@ -131,7 +131,7 @@ cudaError_t launch_accept(const RowMap& m, const Model& md, KvState& kv,
   ++kv.launches;
   AcceptArgs a{m, cand, kv.best, kv.d_len, kv.d_root, kv.d_err + 1, out.n_accepted,
                out.correction_token, out.greedy, mode};
-  return launch_pdl(accept_kernel, dim3(m.batch), dim3(32), 0, st, a);
+  return launch_pdl(accept_kernel, dim3(m.batch), dim3(32), 0, st, 1, a);
 }
 
 cudaError_t launch_rollback(KvState& kv, const int32_t* new_len,
@@ -142,7 +142,7 @@ cudaError_t launch_rollback(KvState& kv, const int32_t* new_len,
     a.len[b] = new_len[b];
     a.root[b] = new_root[b];
   }
-  return launch_pdl(rollback_kernel, dim3(1), dim3(kMaxBatch), 0, st, a, kv.d_len, kv.d_root,
+  return launch_pdl(rollback_kernel, dim3(1), dim3(kMaxBatch), 0, st, 1, a, kv.d_len, kv.d_root,
                     kv.d_err);
 }
 

@@ -15,13 +15,14 @@ namespace as2d {
 namespace {
 
 // Row sources of one packed matrix: plain concatenation of up to three
-// segments (e.g. q, k, v projections), or gate/up interleaving (tile rows
-// 0..63 from gate rows 64t.., 64..127 from up rows 64t..).
+// segments (e.g. q, k, v projections), or gate/up interleaving: of every 32
+// rows 16 gate rows, then the up rows of the same features, so that one warp
+// of the SwiGLU epilogue holds both.
 struct PackSrc {
   const bf16* seg[3];
   int seg_rows[3];
   int nseg;
-  int interleave;  // 1: gate (seg 0) / up (seg 1) in blocks of 64 rows
+  int interleave;  // 1: gate (seg 0) / up (seg 1) in blocks of 16 rows
   int n_rows;      // logical rows
   int K;
 };
@@ -34,8 +35,8 @@ __global__ void __launch_bounds__(256) pack_kernel(PackSrc s, bf16* __restrict__
     const int R = tile * 128 + r;
     const bf16* src = nullptr;
     if (s.interleave) {
-      const int f = (R >> 7) * 64 + (R & 63);
-      if (f < s.seg_rows[0]) src = s.seg[(R & 64) ? 1 : 0] + (size_t)f * s.K;
+      const int f = (R >> 5) * 16 + (R & 15);
+      if (f < s.seg_rows[0]) src = s.seg[(R & 16) ? 1 : 0] + (size_t)f * s.K;
     } else if (R < s.n_rows) {
       int rr = R, q = 0;
       while (q < s.nseg - 1 && rr >= s.seg_rows[q]) rr -= s.seg_rows[q++];

@@ -4,7 +4,7 @@
 
 namespace as2d {
 
-cudaError_t tc_gemm_part(int nb, const CUtensorMap& x, const TcParams& p, cudaStream_t st) {
+cudaError_t tc_gemm_part(int nb, const TcMaps& x, const TcParams& p, cudaStream_t st) {
   return tc_gemm_dispatch<TC_PART>(nb, x, p, st);
 }
 

@@ -3,8 +3,7 @@
 
 namespace as2d {
 
-cudaError_t tc_gemm_swiglu(int nb, const CUtensorMap& x, const TcParams& p,
-                          cudaStream_t st) {
+cudaError_t tc_gemm_swiglu(int nb, const TcMaps& x, const TcParams& p, cudaStream_t st) {
   return tc_gemm_dispatch<TC_SWIGLU>(nb, x, p, st);
 }
 
