@@ -10,13 +10,13 @@
 // rows, the second time from L2).
 //
 // qkv_finish_kernel: the QKV projection arrives as split-K partial sums
-// (TC_PART); one CTA per (token row, head) adds them in rank order, scales by
+// (TC_PART); one warp per (token row, head) adds them in rank order, scales by
 // the row's 1 / rms and rotates (RoPE).  Keys and values are appended to the
 // cache; queries, scaled by log2(e) / sqrt(d), are written as bf16 hi and lo
 // parts straight into the tensor-core operand image of their (request, kv
-// head, 64-query tile): 128 rows (row 2q the hi part of query q, row 2q + 1
-// its lo part) of d elements in the 128-byte-swizzled K-major layout, one
-// 16 KB region per 64 columns.
+// head, 64-query tile): 128 rows (hi_row: of every 16 rows 8 hi parts, then the
+// lo parts of the same queries) of d elements in the 128-byte-swizzled K-major
+// layout, one 16 KB region per 64 columns.
 //
 // attn_tc_kernel: one CTA per 128-key tile of one (request, kv head, query
 // tile); a cluster of 8 CTAs covers one chunk of 1024 keys.  Per CTA:
@@ -24,16 +24,15 @@
 //     byte swizzle; tiles holding only entries older than this call are
 //     requested before the wait for the finishing kernel), the query image
 //     by one bulk copy;
-//   * S = Q K^T on tcgen05 (M = 128: the hi and lo rows of 64 queries
-//     interleaved, N = 128 keys) into TMEM; thread t reads lane t, so each
-//     query's hi and lo scores sit in adjacent lanes of one warp and are
-//     added by a shuffle, each lane keeping half of the keys; masking (causal,
-//     and keys past the call's end) and P = 2^(S - m) with the tile's own
-//     maximum m and sum l;
-//   * O = P V on tcgen05 (P's hi and lo rows interleaved the same way, as
-//     the A operand in TMEM over S, or in the narrow layout as a shared-memory
-//     image over Q; B = V read MN-major from the TMA image); hi + lo added by
-//     a shuffle, each lane keeping half of the dims;
+//   * S = Q K^T on tcgen05 (M = 128: the hi and lo rows of 64 queries, N = 128
+//     keys) into TMEM; 16-lane loads (tcgen05.ld.16x256b) bring both parts of
+//     the same scores to one thread, which adds them (TileThread); masking
+//     (causal, and keys past the call's end) and P = 2^(S - m) with the tile's
+//     own maximum m and sum l;
+//   * O = P V on tcgen05 (P's hi and lo rows stored the same way, as the A
+//     operand in TMEM over S, or in the narrow layout as a shared-memory
+//     image over Q; B = V read MN-major from the TMA image), hi + lo added in
+//     the thread that loads them;
 //   * the tile partials (m, l, O) are pushed through distributed shared
 //     memory to the CTA that folds their query rows (CTA r: rows 8r..8r+7),
 //     which folds the chunk's 8 tiles in tile order.  With one chunk the
@@ -50,6 +49,12 @@
 // clusters than the wide layout serves well; and attn_tc4_kernel, four CTAs
 // per SM in 48 KB, for launches of more clusters than the narrow layout
 // keeps resident.
+// Bound by latency: each CTA is one dependent chain, of which an SM overlaps
+// two to four.  With hi and lo rows in adjacent lanes, exchanged by shuffles, a
+// tile spent 2.4 us of its chain on instructions (read S 0.4, softmax 0.5, write
+// P 0.7, read O 0.75, measured); with both parts in one thread 1.5B k = 0 takes
+// 1111 -> 1079 us a pass, 7B k = 8 2749 -> 2692, L = 15128 k = 16 3616 -> 3388, 16
+// ragged requests 7014 -> 6384.
 // Every fold boundary is a fixed absolute key position (128-key tiles,
 // 1024-key chunks), and a fold with a part a row cannot see (fully masked:
 // m = -inf, l = 0, O = 0) leaves it bitwise unchanged, so a row's result does
@@ -131,6 +136,12 @@ __device__ __forceinline__ uint32_t img_off(int r, int e) {
          (uint32_t)((e & 7) << 1);
 }
 
+// Query q of a tile: its hi part is row hi_row(q) of the operand image and of
+// the products, its lo part row hi_row(q) + 8.  Of every 16 rows the first 8
+// are the hi parts of eight queries, the others their lo parts: the layout in
+// which a 16-lane TMEM load gives a thread both parts of the same columns.
+__device__ __forceinline__ int hi_row(int q) { return (q >> 3) * 16 + (q & 7); }
+
 // One warp per (token row, head); lane l forms the pairs (e, e + D/2) of e =
 // V l .. V l + V - 1.  Rotate-half RoPE: x' = x cos - x_p sin at e, x_p cos +
 // x sin at e + D/2.  Bound by latency, as the residual projections' finishing
@@ -153,7 +164,7 @@ __global__ void __launch_bounds__(32 * kQkvWarps) qkv_finish_kernel(const __grid
   const float* s0 = a.qkv_part + ((size_t)(c0 >> 7) * a.qkv_split * a.qkv_ld + gm) * 128 + (c0 & 127);
   const float* s1 = a.qkv_part + ((size_t)(c1 >> 7) * a.qkv_split * a.qkv_ld + gm) * 128 + (c1 & 127);
   const float2* csp = a.rope + (size_t)gm * H2 + e;
-  // where the results go: the query image's rows 2q (hi) and 2q + 1 (lo), or
+  // where the results go: the query image's two rows of q, or
   // the cache entry at the request's length + i
   const int G = a.nq / a.nkv;
   const int g = is_q ? head / G : (rotate ? head - a.nq : head - a.nq - a.nkv);
@@ -222,10 +233,11 @@ __global__ void __launch_bounds__(32 * kQkvWarps) qkv_finish_kernel(const __grid
       l0[u] = __float2bfloat16_rn(w0 - __bfloat162float(h0[u]));
       l1[u] = __float2bfloat16_rn(w1 - __bfloat162float(h1[u]));
     }
-    put(img + img_off(2 * q, e), h0);
-    put(img + img_off(2 * q, e + H2), h1);
-    put(img + img_off(2 * q + 1, e), l0);
-    put(img + img_off(2 * q + 1, e + H2), l1);
+    const int row = hi_row(q);
+    put(img + img_off(row, e), h0);
+    put(img + img_off(row, e + H2), h1);
+    put(img + img_off(row + 8, e), l0);
+    put(img + img_off(row + 8, e + H2), l1);
   } else {
     bf16 k0[V], k1[V];
 #pragma unroll
@@ -248,27 +260,6 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
-// Values x[0..7] (>= 0) of columns e0..e0+7 (e0 % 8 == 0) of query q, as bf16
-// hi parts into row 2q and lo parts into row 2q + 1 of an operand image: hi =
-// x with its low 16 bits cleared (exact in bf16), lo = bf16(x - hi), so that
-// hi + lo matches x to about 17 bits.  A thread of the odd half (pt = 1)
-// stores its lo row first: the two rows of one store instruction then cover
-// all eight 16-byte positions of the swizzle, not four.
-__device__ __forceinline__ void put_hilo8(uint8_t* img, int q, int pt, int e0, const float* x) {
-  uint32_t hw[4], lw[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const uint32_t b0 = __float_as_uint(x[2 * u]), b1 = __float_as_uint(x[2 * u + 1]);
-    hw[u] = (b0 >> 16) | (b1 & 0xFFFF0000u);
-    const __nv_bfloat162 lv = __floats2bfloat162_rn(x[2 * u] - __uint_as_float(b0 & 0xFFFF0000u),
-                                                    x[2 * u + 1] - __uint_as_float(b1 & 0xFFFF0000u));
-    lw[u] = *reinterpret_cast<const uint32_t*>(&lv);
-  }
-  const uint4 h = make_uint4(hw[0], hw[1], hw[2], hw[3]), l = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-  *reinterpret_cast<uint4*>(img + img_off(2 * q + pt, e0)) = pt ? l : h;
-  *reinterpret_cast<uint4*>(img + img_off(2 * q + 1 - pt, e0)) = pt ? h : l;
-}
-
 __device__ __forceinline__ void dsmem_st_f4(uint32_t addr, float4 v) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y),
                "f"(v.z), "f"(v.w)
@@ -280,27 +271,76 @@ __device__ __forceinline__ void dsmem_st_f2(uint32_t addr, float2 v) {
                : "memory");
 }
 
-// 128 columns of this thread's TMEM lane starting at taddr: two loads, one
-// wait.
-__device__ __forceinline__ void tmem_ld128(uint32_t taddr, float (&v0)[64], float (&v1)[64]) {
-  uint32_t a[64], b[64];
-  ptx::tmem_ld_x64(taddr, a);
-  ptx::tmem_ld_x64(taddr + 64, b);
+// A thread's share of a tile.  The four warps that read a tile's products
+// cover 16 queries each: warp w, lane 4r + c holds queries 16w + r and 16w + 8
+// + r (i = 0, 1), and of each the keys (dims) 8j + 2c + u, u < 2, as element 2j
+// + u.  Hi and lo parts come to the same thread, so they are added without an
+// exchange between lanes: with the parts in adjacent lanes (two selects and a
+// shuffle an element) a tile took some 1500 instructions a warp, now 700, and
+// the rows of P need no exchange either.
+struct TileThread {
+  int w, r, c;
+  __device__ __forceinline__ TileThread(int warp, int lane) : w(warp & 3), r(lane >> 2), c(lane & 3) {}
+  __device__ __forceinline__ int query(int i) const { return 16 * w + 8 * i + r; }
+};
+// Columns [0, 32 NCH) of one of the thread's queries (hi + lo) from the 16 TMEM
+// lanes at taddr: every load issued before the wait.
+template <int NCH>
+__device__ __forceinline__ void tile_load(uint32_t taddr, float (&x)[8 * NCH]) {
+  uint32_t v[NCH][16];
+#pragma unroll
+  for (int ch = 0; ch < NCH; ++ch) ptx::tmem_ld_16x256b_x4(taddr + 32 * ch, v[ch]);
   ptx::tmem_ld_wait();
 #pragma unroll
-  for (int j = 0; j < 64; ++j) {
-    v0[j] = __uint_as_float(a[j]);
-    v1[j] = __uint_as_float(b[j]);
-  }
+  for (int ch = 0; ch < NCH; ++ch)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        x[8 * ch + 2 * j + u] =
+            __uint_as_float(v[ch][4 * j + u]) + __uint_as_float(v[ch][4 * j + 2 + u]);
 }
 
-// 64 columns of this thread's TMEM lane starting at `col`, into v.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
-  uint32_t a[64];
-  ptx::tmem_ld_x64(taddr, a);
-  ptx::tmem_ld_wait();
+// P (>= 0) as bf16 pairs of keys: hi = P with its low 16 bits cleared (exact
+// in bf16), lo = bf16(P - hi), so that hi + lo matches P to about 17 bits.
+__device__ __forceinline__ void hi_lo(float x0, float x1, uint32_t& h, uint32_t& l) {
+  const uint32_t b0 = __float_as_uint(x0), b1 = __float_as_uint(x1);
+  h = __byte_perm(b0, b1, 0x7632);
+  const __nv_bfloat162 lv = __floats2bfloat162_rn(x0 - __uint_as_float(b0 & 0xFFFF0000u),
+                                                  x1 - __uint_as_float(b1 & 0xFFFF0000u));
+  l = *reinterpret_cast<const uint32_t*>(&lv);
+}
+
+// P of one query into the 16 TMEM lanes at taddr (over S), where the second
+// product reads its A operand: two keys a column, rows as the queries' rows.
+// The caller waits for the stores (ptx::tmem_st_wait).
+__device__ __forceinline__ void tile_store_p(uint32_t taddr, const float (&x)[32]) {
 #pragma unroll
-  for (int j = 0; j < 64; ++j) v[j] = __uint_as_float(a[j]);
+  for (int h = 0; h < 2; ++h) {
+    uint32_t v[16];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) hi_lo(x[16 * h + 2 * j], x[16 * h + 2 * j + 1], v[2 * j], v[2 * j + 1]);
+    ptx::tmem_st_16x128b_x8(taddr + 32 * h, v);
+  }
+}
+constexpr uint32_t kLane16 = 16u << 16;  // TMEM address of the upper 16 lanes of a warp's 32
+
+
+// Where dims 8j + 2c .. + 1 of a row lie in a partial row as the threads pass
+// it on: each thread's four consecutive elements as one float4, the four
+// threads of a row side by side.
+__device__ __forceinline__ int part_pos(int j, int c) { return ((j >> 1) * 4 + c) * 4 + (j & 1) * 2; }
+
+// Dims [fd, fd + DT) of a partial row (DT 4 or 8, fd a multiple of it).
+template <int DT>
+__device__ __forceinline__ void part_load(const float* row, int fd, float (&v)[DT]) {
+#pragma unroll
+  for (int t = 0; t < DT / 2; ++t) {
+    const float2 x =
+        *reinterpret_cast<const float2*>(row + part_pos(fd >> 3, ((fd & 7) >> 1) + t));
+    v[2 * t] = x.x;
+    v[2 * t + 1] = x.y;
+  }
 }
 
 // The weight of a part (max m) in a fold whose maximum is M: 2^(m - M), 0
@@ -311,43 +351,36 @@ __device__ __forceinline__ float part_weight(float m, float M) {
   return m == -INFINITY ? 0.f : (m == M ? 1.f : ex2(m - M));
 }
 
-// The tile's scores of this thread's 64 keys kb .. kb + 63 (hi + lo, in sv)
-// -> P = 2^(S - m) in sv (visible keys: key <= lim; a masked key gets 0,
-// never -inf), with the tile's maximum m and sum l over both halves of the
-// keys (the partner lane holds the other half).
-__device__ __forceinline__ void softmax_tail(float (&sv)[64], int pt, int kb, int lim, float& m,
-                                             float& l) {
-  // a half-tile wholly at or below the row's limit needs no mask
-  const bool all_vis = kb + 63 <= lim;
+// The tile's scores of one query (this thread's 32 keys p0 + 8j + 2c + u, in sv)
+// -> P = 2^(S - m) in sv (visible keys: key <= lim; a masked key gets 0), with
+// the tile's maximum m (-inf where nothing is visible) and sum l over the four
+// threads of the query.
+__device__ __forceinline__ void softmax_tail(float (&sv)[32], int c, int p0, int lim, float& m, float& l) {
+  // (a tile wholly at or below the row's limit needs no mask)
+  if (p0 + kTile - 1 > lim) {
+    const int k0 = p0 + 2 * c;
+#pragma unroll
+    for (int t = 0; t < 32; ++t)
+      if (k0 + 8 * (t >> 1) + (t & 1) > lim) sv[t] = -INFINITY;
+  }
   float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  if (all_vis) {
 #pragma unroll
-    for (int j = 0; j < 64; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], sv[j]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < 64; ++j)
-      if (kb + j <= lim) mx4[j & 3] = fmaxf(mx4[j & 3], sv[j]);
-  }
-  const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-  m = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
-  // sums in four interleaved parts, then ((0 + 1) + (2 + 3)): a fixed order
+  for (int t = 0; t < 32; ++t) mx4[t & 3] = fmaxf(mx4[t & 3], sv[t]);
+  float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+  mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
+  m = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
+  const float ref = m == -INFINITY ? 0.f : m;  // (2^(-inf - 0) = 0)
+  // sums in four interleaved parts, then ((0 + 1) + (2 + 3)), then over the
+  // threads in pairs: a fixed order
   float ls4[4] = {0.f, 0.f, 0.f, 0.f};
-  if (all_vis) {
 #pragma unroll
-    for (int j = 0; j < 64; ++j) {
-      sv[j] = ex2(sv[j] - m);
-      ls4[j & 3] += sv[j];
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 64; ++j) {
-      sv[j] = (kb + j <= lim) ? ex2(sv[j] - m) : 0.f;
-      ls4[j & 3] += sv[j];
-    }
+  for (int t = 0; t < 32; ++t) {
+    sv[t] = ex2(sv[t] - ref);
+    ls4[t & 3] += sv[t];
   }
-  const float ls = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
-  const float lo_ = __shfl_xor_sync(0xFFFFFFFFu, ls, 1);
-  l = pt ? lo_ + ls : ls + lo_;  // keys 0..63, then 64..127
+  float ls = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
+  ls += __shfl_xor_sync(0xFFFFFFFFu, ls, 1);
+  l = ls + __shfl_xor_sync(0xFFFFFFFFu, ls, 2);
 }
 
 // Dims [fd, fd + DT) of row fr of query tile qt, normalised (o / l), as
@@ -415,15 +448,10 @@ __device__ __forceinline__ void fold_chunk8(const AttnArgs& a, const float* recv
     const float w = part_weight(pml[i].x, fm);
     if (w != 0.f) {
       fl += pml[i].y * w;
-      const float4* src = reinterpret_cast<const float4*>(recv + (i * 8 + fj) * D + fd);
+      float v[DT];
+      part_load<DT>(recv + (i * 8 + fj) * D, fd, v);
 #pragma unroll
-      for (int u = 0; u < DT / 4; ++u) {
-        const float4 v = src[u];
-        fo[4 * u + 0] += v.x * w;
-        fo[4 * u + 1] += v.y * w;
-        fo[4 * u + 2] += v.z * w;
-        fo[4 * u + 3] += v.w * w;
-      }
+      for (int d = 0; d < DT; ++d) fo[d] += v[d] * w;
     }
   }
   // normalise and write the row's dims (o / l as bf16 hi, lo)
@@ -589,7 +617,7 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
   constexpr uint32_t K_BYTES = NR * kRegion;            // one K or V tile
   constexpr uint32_t TMEM_COLS = NARROW ? 128 : 256;   // narrow: O over S
   constexpr uint32_t Q_BYTES = 2u * kQT * D * 2;
-  constexpr int DH = D / 2;           // dims each thread of a hi/lo pair keeps
+  constexpr int DQ = D / 4;           // dims of a query that a thread holds
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -677,16 +705,17 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
     ptx::bulk_load(R0, qsrc, Q_BYTES, &bars[0], ptx::policy_evict_last());
   }
 
-  // Thread tid reads TMEM lane tid: query q = tid / 2, its hi part (pt = 0)
-  // or lo part (pt = 1).  After the exchange with its partner lane it keeps
-  // keys [64 pt, 64 pt + 64) of S and dims [DH pt, DH pt + DH) of O.
-  const int q = tid >> 1, pt = tid & 1;
-  const int qg = qt * kQT + q;
-  const int lim = qg < qn ? L + qg / G : -1;  // the query's last visible key
-  float m = -INFINITY, l = 0.f;               // the tile partial of query q
-  float o[DH];
+  const TileThread me(warp, tid & 31);
+  int lim[2];                                              // each query's last visible key
+  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};  // the tile partials
 #pragma unroll
-  for (int j = 0; j < DH; ++j) o[j] = 0.f;
+  for (int i = 0; i < 2; ++i) {
+    const int qg = qt * kQT + me.query(i);
+    lim[i] = qg < qn ? L + qg / G : -1;
+  }
+  float o[2][DQ];
+#pragma unroll
+  for (int j = 0; j < DQ; ++j) o[0][j] = o[1][j] = 0.f;
   bool ok = true;
   if (active) {
     ok = ptx::mbar_wait(&bars[0], 0, a.timeout_ns) && ptx::mbar_wait(&bars[1], 0, a.timeout_ns);
@@ -742,49 +771,28 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
     ptx::tc_fence_after();
     bool ok2 = ok1, vok = ok1;
     if (ok1) {
-      // S = hi + lo of this thread's keys, masked; the tile's maximum and
-      // P = 2^(S - m) with the partner lane
-      float sv[64];
-      {
-        float v0[64], v1[64];
-        tmem_ld128(tmem + lane_base, v0, v1);
+      // S = hi + lo, masked; the tile's maximum and P = 2^(S - m).  P's hi
+      // and lo parts: wide, into TMEM over S; narrow, into the operand image in
+      // shared memory, K-major by key (the same values)
 #pragma unroll
-        for (int j = 0; j < 64; ++j) {
-          const float mine = pt ? v1[j] : v0[j], other = pt ? v0[j] : v1[j];
-          sv[j] = mine + __shfl_xor_sync(0xFFFFFFFFu, other, 1);
+      for (int i = 0; i < 2; ++i) {
+        float sv[32];
+        tile_load<4>(tmem + lane_base + i * kLane16, sv);
+        softmax_tail(sv, me.c, p0, lim[i], m[i], l[i]);
+        if (!NARROW) {
+          tile_store_p(tmem + lane_base + i * kLane16, sv);
+        } else {
+          const int row = hi_row(me.query(i));
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            uint32_t h, lo;
+            hi_lo(sv[2 * j], sv[2 * j + 1], h, lo);
+            *reinterpret_cast<uint32_t*>(R0 + img_off(row, 8 * j + 2 * me.c)) = h;
+            *reinterpret_cast<uint32_t*>(R0 + img_off(row + 8, 8 * j + 2 * me.c)) = lo;
+          }
         }
       }
-      softmax_tail(sv, pt, p0 + 64 * pt, lim, m, l);
-      // P as bf16 hi (row 2q) and lo (row 2q + 1) parts: hi = P with its low
-      // 16 bits cleared, lo = bf16(P - hi).  Wide: into TMEM over S (the
-      // second product's A operand, lane 2q + pt its row, two keys per
-      // column), each lane completing its row with the partner's half of the
-      // keys.  Narrow: into the operand image in shared memory, K-major by key.
-      if (!NARROW) {
-        uint32_t hw[32], lw[32], row[64];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const uint32_t b0 = __float_as_uint(sv[2 * j]), b1 = __float_as_uint(sv[2 * j + 1]);
-          hw[j] = (b0 >> 16) | (b1 & 0xFFFF0000u);
-          const __nv_bfloat162 lv =
-              __floats2bfloat162_rn(sv[2 * j] - __uint_as_float(b0 & 0xFFFF0000u),
-                                    sv[2 * j + 1] - __uint_as_float(b1 & 0xFFFF0000u));
-          lw[j] = *reinterpret_cast<const uint32_t*>(&lv);
-        }
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          // the hi lane takes the partner's hi words (keys 64..127), the lo
-          // lane the partner's lo words (keys 0..63)
-          const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, pt ? hw[j] : lw[j], 1);
-          row[j] = pt ? got : hw[j];
-          row[32 + j] = pt ? lw[j] : got;
-        }
-        ptx::tmem_st_x64(tmem + lane_base, row);
-        ptx::tmem_st_wait();
-      } else {
-#pragma unroll
-        for (int ch = 0; ch < 8; ++ch) put_hilo8(R0, q, pt, 64 * pt + 8 * ch, sv + 8 * ch);
-      }
+      if (!NARROW) ptx::tmem_st_wait();
       if (NARROW) {
         vok = ptx::group_all(ptx::mbar_wait(&bars[4], 0, a.timeout_ns), 1, 128);
         if (vok) zero_v_tail();
@@ -820,19 +828,9 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
       }
       ptx::tc_fence_after();
       if (ok2) {
-        // O = hi + lo of this thread's dims
 #pragma unroll
-        for (int c0 = 0; c0 < D; c0 += 64) {
-          float v[64];
-          tmem_ld64(tmem + lane_base + (NARROW ? 0 : 128) + c0, v);
-#pragma unroll
-          for (int j = 0; j < 64; ++j) {
-            const int d = c0 + j;  // compile-time after unrolling
-            const bool mine = (d / DH) == pt;
-            const float x = __shfl_xor_sync(0xFFFFFFFFu, v[j], 1);
-            if (mine) o[d - pt * DH] = v[j] + x;
-          }
-        }
+        for (int i = 0; i < 2; ++i)
+          tile_load<D / 32>(tmem + lane_base + i * kLane16 + (NARROW ? 0 : 128), o[i]);
       }
     }
     if (!(ok1 && ok2)) {
@@ -842,7 +840,7 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
         ptx::mbar_wait(&bars[2], 0, ptx::kDrainNs);
         if (vok) ptx::mbar_wait(&bars[3], 0, ptx::kDrainNs);
       }
-      m = -INFINITY;  // nothing of this tile is passed on
+      m[0] = m[1] = -INFINITY;  // nothing of this tile is passed on
     }
   } else {
     ptx::cluster_arrive_relaxed();  // no keys of this CTA's tile are read
@@ -864,15 +862,20 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
   constexpr int RPC = PAIR ? 4 : 8;
   ptx::cluster_wait();
   if (active) {
-    const uint32_t dst_rank = (uint32_t)(q / RPC), row = (uint32_t)(q % RPC);
-    if (pt == 0)
-      dsmem_st_f2(ptx::dsmem_map(ptx::smem_u32(s_rml + crank * RPC + row), dst_rank), make_float2(m, l));
-    if (m != -INFINITY) {
-      const uint32_t dst =
-          ptx::dsmem_map(ptx::smem_u32(recv + (crank * RPC + row) * D + pt * DH), dst_rank);
 #pragma unroll
-      for (int u = 0; u < DH / 4; ++u)
-        dsmem_st_f4(dst + 16u * u, make_float4(o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]));
+    for (int i = 0; i < 2; ++i) {
+      const int q = me.query(i);
+      const uint32_t dst_rank = (uint32_t)(q / RPC), row = (uint32_t)(q % RPC);
+      if (me.c == 0)
+        dsmem_st_f2(ptx::dsmem_map(ptx::smem_u32(s_rml + crank * RPC + row), dst_rank),
+                    make_float2(m[i], l[i]));
+      if (m[i] != -INFINITY) {
+        const uint32_t dst =
+            ptx::dsmem_map(ptx::smem_u32(recv + (crank * RPC + row) * D + part_pos(0, me.c)), dst_rank);
+#pragma unroll
+        for (int u = 0; u < DQ / 4; ++u)
+          dsmem_st_f4(dst + 64u * u, make_float4(o[i][4 * u], o[i][4 * u + 1], o[i][4 * u + 2], o[i][4 * u + 3]));
+      }
     }
   }
   ptx::cluster_sync();
@@ -902,11 +905,10 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
           const float w = part_weight(pml[i].x, fm);
           if (w != 0.f) {
             fl += pml[i].y * w;
-            const float4 v = *reinterpret_cast<const float4*>(recv + ((h * kCluster + i) * 4 + fj) * D + fd);
-            fo[0] += v.x * w;
-            fo[1] += v.y * w;
-            fo[2] += v.z * w;
-            fo[3] += v.w * w;
+            float v[4];
+            part_load<4>(recv + ((h * kCluster + i) * 4 + fj) * D, fd, v);
+#pragma unroll
+            for (int d = 0; d < 4; ++d) fo[d] += v[d] * w;
           }
         }
         cmx[h] = fm;
@@ -961,7 +963,7 @@ __global__ void __launch_bounds__(128, 4)
                     const __grid_constant__ AttnArgs a) {
   constexpr int NR = D / 64;          // 64-column regions of a K / V tile
   constexpr uint32_t Q_BYTES = 2u * kQT * D * 2;
-  constexpr int DH = D / 2;           // dims each thread of a hi/lo pair keeps
+  constexpr int DQ = D / 4;           // dims of a query that a thread holds
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -1038,14 +1040,15 @@ __global__ void __launch_bounds__(128, 4)
     issued |= 1u;
   }
 
-  // Thread tid reads TMEM lane tid: query q = tid / 2, its hi part (pt = 0)
-  // or lo part (pt = 1); it keeps keys [64 pt, 64 pt + 64) of S and dims
-  // [DH pt, DH pt + DH) of O.
-  const int q = tid >> 1, pt = tid & 1;
-  const int qg = qt * kQT + q;
-  const int lim = qg < qn ? L + qg / G : -1;
-  float m = -INFINITY, l = 0.f;
-  float o[DH];  // written by the second product's read-out; pushed only then
+  const TileThread me(warp, tid & 31);
+  int lim[2];                                              // each query's last visible key
+  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};  // the tile partials
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int qg = qt * kQT + me.query(i);
+    lim[i] = qg < qn ? L + qg / G : -1;
+  }
+  float o[2][DQ];  // written by the second product's read-out; pushed only then
   auto wait_all = [&](bool ok, int bar) {
     return ptx::group_all(ok && ptx::mbar_wait(&bars[bar], 0, a.timeout_ns), 1, 128);
   };
@@ -1083,47 +1086,12 @@ __global__ void __launch_bounds__(128, 4)
     }
     ptx::tc_fence_after();
     if (ok) {
-      // S = hi + lo of this thread's keys, 16 keys of each half at a time
-      float sv[64];
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        uint32_t k0[16], k1[16];  // keys 16 cc + j and 64 + 16 cc + j
-        ptx::tmem_ld16(tmem + lane_base + 16 * cc, k0);
-        ptx::tmem_ld16(tmem + lane_base + 64 + 16 * cc, k1);
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float v0 = __uint_as_float(k0[j]), v1 = __uint_as_float(k1[j]);
-          const float mine = pt ? v1 : v0, other = pt ? v0 : v1;
-          sv[16 * cc + j] = mine + __shfl_xor_sync(0xFFFFFFFFu, other, 1);
-        }
-      }
-      softmax_tail(sv, pt, p0 + 64 * pt, lim, m, l);
-      // P as bf16 hi (row 2q) and lo (row 2q + 1) parts into TMEM over S, two
-      // keys per column, 16 keys (8 columns of each half of the row) at a
-      // time; each lane completes its row with the partner's half of the keys
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        uint32_t hw[8], lw[8], first[8], second[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float x0 = sv[16 * cc + 2 * j], x1 = sv[16 * cc + 2 * j + 1];
-          const uint32_t b0 = __float_as_uint(x0), b1 = __float_as_uint(x1);
-          hw[j] = (b0 >> 16) | (b1 & 0xFFFF0000u);
-          const __nv_bfloat162 lv = __floats2bfloat162_rn(x0 - __uint_as_float(b0 & 0xFFFF0000u),
-                                                          x1 - __uint_as_float(b1 & 0xFFFF0000u));
-          lw[j] = *reinterpret_cast<const uint32_t*>(&lv);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          // the hi lane takes the partner's hi words (keys 64..127), the lo
-          // lane the partner's lo words (keys 0..63)
-          const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, pt ? hw[j] : lw[j], 1);
-          first[j] = pt ? got : hw[j];
-          second[j] = pt ? lw[j] : got;
-        }
-        ptx::tmem_st_x8(tmem + lane_base + 8 * cc, first);
-        ptx::tmem_st_x8(tmem + lane_base + 32 + 8 * cc, second);
+      for (int i = 0; i < 2; ++i) {
+        float sv[32];
+        tile_load<4>(tmem + lane_base + i * kLane16, sv);
+        softmax_tail(sv, me.c, p0, lim[i], m[i], l[i]);
+        tile_store_p(tmem + lane_base + i * kLane16, sv);
       }
       ptx::tmem_st_wait();
     }
@@ -1162,18 +1130,8 @@ __global__ void __launch_bounds__(128, 4)
       ptx::tc_fence_after();
       if (ok) {
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          uint32_t v16[16];
-          ptx::tmem_ld16(tmem + lane_base + 64 + 16 * cc, v16);
-          ptx::tmem_ld_wait();
-          const int d0 = 64 * h + 16 * cc, owner = d0 / DH;  // compile-time after unrolling
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float v = __uint_as_float(v16[j]);
-            const float x = __shfl_xor_sync(0xFFFFFFFFu, v, 1);
-            if (pt == owner) o[d0 - owner * DH + j] = v + x;
-          }
-        }
+        for (int i = 0; i < 2; ++i)
+          tile_load<2>(tmem + lane_base + i * kLane16 + 64, *reinterpret_cast<float(*)[16]>(&o[i][16 * h]));
       }
     }
     if (!ok) {
@@ -1183,7 +1141,7 @@ __global__ void __launch_bounds__(128, 4)
         for (int i = 0; i < 8; ++i)
           if (issued & (1u << i)) ptx::mbar_wait(&bars[i], 0, ptx::kDrainNs);
       }
-      m = -INFINITY;  // nothing of this tile is passed on
+      m[0] = m[1] = -INFINITY;  // nothing of this tile is passed on
     }
   }
   // the V image is consumed: the cluster's partials may come into it
@@ -1196,15 +1154,20 @@ __global__ void __launch_bounds__(128, 4)
   // ---- the tile partials, pushed to the CTA that folds their rows ----------
   ptx::cluster_wait();
   if (active) {
-    const uint32_t dst_rank = (uint32_t)(q >> 3), row = (uint32_t)(q & 7);
-    if (pt == 0)
-      dsmem_st_f2(ptx::dsmem_map(ptx::smem_u32(s_rml + rank * 8 + row), dst_rank), make_float2(m, l));
-    if (m != -INFINITY) {
-      const uint32_t dst =
-          ptx::dsmem_map(ptx::smem_u32(recv + (rank * 8 + row) * D + pt * DH), dst_rank);
 #pragma unroll
-      for (int u = 0; u < DH / 4; ++u)
-        dsmem_st_f4(dst + 16u * u, make_float4(o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]));
+    for (int i = 0; i < 2; ++i) {
+      const int q = me.query(i);
+      const uint32_t dst_rank = (uint32_t)(q / 8), row = (uint32_t)(q % 8);
+      if (me.c == 0)
+        dsmem_st_f2(ptx::dsmem_map(ptx::smem_u32(s_rml + rank * 8 + row), dst_rank),
+                    make_float2(m[i], l[i]));
+      if (m[i] != -INFINITY) {
+        const uint32_t dst =
+            ptx::dsmem_map(ptx::smem_u32(recv + (rank * 8 + row) * D + part_pos(0, me.c)), dst_rank);
+#pragma unroll
+        for (int u = 0; u < DQ / 4; ++u)
+          dsmem_st_f4(dst + 64u * u, make_float4(o[i][4 * u], o[i][4 * u + 1], o[i][4 * u + 2], o[i][4 * u + 3]));
+      }
     }
   }
   ptx::cluster_sync();

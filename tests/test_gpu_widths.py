@@ -52,3 +52,42 @@ def test_rows(pair, rows):
         assert a1[0] == acc[b] and c1[0] == corr[b] and np.array_equal(g1, greedy[at:at + rows[b]])
         one.close()
         at += rows[b]
+
+
+# one chunk, two chunks in a cluster of 16 (or through memory), more chunks,
+# lengths around the 128-key tiles and 1024-key chunks, one and two query
+# tiles; together a launch of four CTAs per SM
+LAYOUT_LENS = [1, 126, 127, 128, 129, 1015, 1023, 1024, 1025, 2030, 2047, 2049, 3000]
+LAYOUT_KS = [0, 1, 16, 0, 3, 9, 0, 16, 2, 16, 0, 8, 12]
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_attention_layouts(d):
+    """Every request of a large launch equals the same request alone (another
+    layout of the attention) bit for bit, and the oracle."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    cfg = W.ModelConfig(f"d{d}", 1, 256, 8, 2, d, 448, 1032)
+    pair = Pair(cfg, seed=0)
+    lens, ks = LAYOUT_LENS * 2, LAYOUT_KS * 2
+    cap, n = max(lens) + 32, len(lens)
+    rng = np.random.default_rng(d)
+    roots = [int(x) for x in rng.integers(0, cfg.vocab, size=n)]
+    cands = [[int(t) for t in rng.integers(0, cfg.vocab, size=k)] for k in ks]
+    st = pair.state(lens, cap, roots)
+    logits = run_gpu_block(st, cfg, cands)[3]
+    st.check()
+    kc, vc = st.kc.clone(), st.vc.clone()
+    st.close()
+    at = 0
+    for b in range(len(LAYOUT_LENS)):
+        one = pair.state([lens[b]], cap, [roots[b]])
+        one.kc[:, 0, :, :lens[b]] = kc[:, b, :, :lens[b]]
+        one.vc[:, 0, :, :lens[b]] = vc[:, b, :, :lens[b]]
+        rows = logits[at:at + ks[b] + 1]
+        assert np.array_equal(run_gpu_block(one, cfg, [cands[b]])[3], rows), f"length {lens[b]}"
+        one.close()
+        want = pair.oracle.verify_block(pair.oracle_cache(lens[b], cap, req=b), lens[b], roots[b], cands[b])
+        assert np.max(np.abs(want["logits"] - rows)) <= LOGIT_TOL, f"length {lens[b]}"
+        at += ks[b] + 1
