@@ -326,22 +326,11 @@ __device__ __forceinline__ void tile_store_p(uint32_t taddr, const float (&x)[32
 constexpr uint32_t kLane16 = 16u << 16;  // TMEM address of the upper 16 lanes of a warp's 32
 
 
-// Where dims 8j + 2c .. + 1 of a row lie in a partial row as the threads pass
-// it on: each thread's four consecutive elements as one float4, the four
-// threads of a row side by side.
-__device__ __forceinline__ int part_pos(int j, int c) { return ((j >> 1) * 4 + c) * 4 + (j & 1) * 2; }
-
-// Dims [fd, fd + DT) of a partial row (DT 4 or 8, fd a multiple of it).
-template <int DT>
-__device__ __forceinline__ void part_load(const float* row, int fd, float (&v)[DT]) {
-#pragma unroll
-  for (int t = 0; t < DT / 2; ++t) {
-    const float2 x =
-        *reinterpret_cast<const float2*>(row + part_pos(fd >> 3, ((fd & 7) >> 1) + t));
-    v[2 * t] = x.x;
-    v[2 * t + 1] = x.y;
-  }
-}
+// A partial row of O as the threads pass it on: position 16v + 4c + 2w + u
+// holds dim 16v + 8w + 2c + u (each thread's four consecutive elements as one
+// float4, the four threads of a row side by side).  The folds keep that order
+// and write_rows undoes it.
+__device__ __forceinline__ int part_pos(int c) { return 4 * c; }  // of thread c; + 16 v
 
 // The weight of a part (max m) in a fold whose maximum is M: 2^(m - M), 0
 // where m = -inf (nothing of the part is visible to the row), exactly 1 for
@@ -383,36 +372,82 @@ __device__ __forceinline__ void softmax_tail(float (&sv)[32], int c, int p0, int
   l = ls + __shfl_xor_sync(0xFFFFFFFFu, ls, 2);
 }
 
-// Dims [fd, fd + DT) of row fr of query tile qt, normalised (o / l), as
-// bf16 hi and lo parts into the attention output; rows past the call's
-// queries are skipped.
+// Positions [fd, fd + DT) (fd a multiple of DT) of row fr of query tile qt,
+// normalised (o / l), as bf16 hi and lo parts into the attention output; rows
+// past the call's queries are skipped.  The quotients are x r, r = 1 / l, with
+// one correction by their remainder (Markstein's method: within a rounding of
+// the quotient), as eight divisions in a row would hold up the chain.
 template <int D, int DT>
 __device__ __forceinline__ void write_rows(const AttnArgs& a, const float* o_, float Ls, int fr,
                                            int fd, int qt, int qn, int G, int g, int r0) {
+  static_assert(DT == 4 || DT == 8, "one or two threads' elements");
   const int fqg = qt * kQT + fr;
   if (fqg >= qn) return;
   const int i = fqg / G, hq = g * G + (fqg - i * G);
-  const size_t at = (size_t)(r0 + i) * a.nq * D + (size_t)hq * D + fd;
-  uint32_t hw[DT / 2], lw[DT / 2];
+  const float inv = 1.f / Ls;
+  uint32_t hw[2][DT / 4], lw[2][DT / 4];  // [dims 2c .., dims 8 + 2c ..]
 #pragma unroll
   for (int e = 0; e < DT / 2; ++e) {
-    const float v0 = o_[2 * e] / Ls, v1 = o_[2 * e + 1] / Ls;
-    const __nv_bfloat162 hv = __floats2bfloat162_rn(v0, v1);
-    const float2 hf = __bfloat1622float2(hv);
-    const __nv_bfloat162 lv = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
-    hw[e] = *reinterpret_cast<const uint32_t*>(&hv);
-    lw[e] = *reinterpret_cast<const uint32_t*>(&lv);
-  }
+    float v[2];
 #pragma unroll
-  for (int u = 0; u < DT / 8; ++u) {
-    *reinterpret_cast<uint4*>(a.ao + at + 8 * u) =
-        make_uint4(hw[4 * u], hw[4 * u + 1], hw[4 * u + 2], hw[4 * u + 3]);
-    *reinterpret_cast<uint4*>(a.ao + (size_t)a.lo_row * a.nq * D + at + 8 * u) =
-        make_uint4(lw[4 * u], lw[4 * u + 1], lw[4 * u + 2], lw[4 * u + 3]);
+    for (int u = 0; u < 2; ++u) {
+      const float x = o_[2 * e + u] * inv;
+      v[u] = fmaf(fmaf(-x, Ls, o_[2 * e + u]), inv, x);
+    }
+    const __nv_bfloat162 hv = __floats2bfloat162_rn(v[0], v[1]);
+    const float2 hf = __bfloat1622float2(hv);
+    const __nv_bfloat162 lv = __floats2bfloat162_rn(v[0] - hf.x, v[1] - hf.y);
+    hw[e & 1][e >> 1] = *reinterpret_cast<const uint32_t*>(&hv);
+    lw[e & 1][e >> 1] = *reinterpret_cast<const uint32_t*>(&lv);
   }
-  if (DT % 8) {  // four dims
-    *reinterpret_cast<uint2*>(a.ao + at) = make_uint2(hw[0], hw[1]);
-    *reinterpret_cast<uint2*>(a.ao + (size_t)a.lo_row * a.nq * D + at) = make_uint2(lw[0], lw[1]);
+  const size_t at = (size_t)(r0 + i) * a.nq * D + (size_t)hq * D + (fd & ~15) + ((fd & 15) >> 1);
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    bf16* hi = a.ao + at + 8 * w;
+    bf16* lo = hi + (size_t)a.lo_row * a.nq * D;
+    if constexpr (DT == 8) {
+      *reinterpret_cast<uint2*>(hi) = make_uint2(hw[w][0], hw[w][1]);
+      *reinterpret_cast<uint2*>(lo) = make_uint2(lw[w][0], lw[w][1]);
+    } else {
+      *reinterpret_cast<uint32_t*>(hi) = hw[w][0];
+      *reinterpret_cast<uint32_t*>(lo) = lw[w][0];
+    }
+  }
+}
+
+// The fold of NT tile partials (rows at o, `stride` floats apart; their
+// maxima m, -inf for none): o and l relative to the largest, fm.  Every load is
+// issued before the first is used, and parts of weight 0 are dropped by
+// selection (what lies in their place is not read into the sums).  The fold
+// stands at the end of every layer's chain: 1.5 us with a branch for each part
+// and eight divisions; without them 1.5B k = 0 / 8 1069 -> 1058 / 1142 -> 1115 us
+// a pass, 7B k = 8 2699 -> 2689, L = 15128 k = 16 3385 -> 3352.
+template <int NT, int DT>
+__device__ __forceinline__ void fold_tiles(const float* o, int stride, const float2 (&ml)[NT], float& fm,
+                                           float& fl, float (&fo)[DT]) {
+  float4 v[NT][DT / 4];
+#pragma unroll
+  for (int i = 0; i < NT; ++i)
+#pragma unroll
+    for (int u = 0; u < DT / 4; ++u) v[i][u] = reinterpret_cast<const float4*>(o + i * stride)[u];
+  fm = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) fm = fmaxf(fm, ml[i].x);
+  fl = 0.f;
+#pragma unroll
+  for (int e = 0; e < DT; ++e) fo[e] = 0.f;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const float w = part_weight(ml[i].x, fm);
+    const bool on = w != 0.f;
+    fl = on ? fmaf(ml[i].y, w, fl) : fl;
+#pragma unroll
+    for (int u = 0; u < DT / 4; ++u) {
+      fo[4 * u] = on ? fmaf(v[i][u].x, w, fo[4 * u]) : fo[4 * u];
+      fo[4 * u + 1] = on ? fmaf(v[i][u].y, w, fo[4 * u + 1]) : fo[4 * u + 1];
+      fo[4 * u + 2] = on ? fmaf(v[i][u].z, w, fo[4 * u + 2]) : fo[4 * u + 2];
+      fo[4 * u + 3] = on ? fmaf(v[i][u].w, w, fo[4 * u + 3]) : fo[4 * u + 3];
+    }
   }
 }
 
@@ -430,31 +465,18 @@ __device__ __forceinline__ void fold_chunk8(const AttnArgs& a, const float* recv
                                             int r0) {
   constexpr int DT = D / 16;  // dims per thread (8 rows x 16 threads)
   const int tid = threadIdx.x;
-  // ---- fold (thread: query row 8 rank + fj, dims [fd, fd + DT)) ----------
+  // ---- fold (thread: query row 8 rank + fj, positions [fd, fd + DT)) ----------
   const int n_here = min(kCluster, n_tiles - c * kCluster);  // tiles of this chunk with keys
   const int fj = tid >> 4, fr = 8 * (int)rank + fj, fd = DT * (tid & 15);
-  float fm = -INFINITY;
-  float2 pml[kCluster];
+  float fm, fl, fo[DT];
+  {
+    float2 pml[kCluster];
 #pragma unroll
-  for (int i = 0; i < kCluster; ++i) {
-    pml[i] = (i < n_here) ? s_rml[i * 8 + fj] : make_float2(-INFINITY, 0.f);
-    fm = fmaxf(fm, pml[i].x);
+    for (int i = 0; i < kCluster; ++i)
+      pml[i] = (i < n_here) ? s_rml[i * 8 + fj] : make_float2(-INFINITY, 0.f);
+    fold_tiles<kCluster, DT>(recv + fj * D + fd, 8 * D, pml, fm, fl, fo);
   }
-  float fl = 0.f, fo[DT];
-#pragma unroll
-  for (int e = 0; e < DT; ++e) fo[e] = 0.f;
-#pragma unroll
-  for (int i = 0; i < kCluster; ++i) {
-    const float w = part_weight(pml[i].x, fm);
-    if (w != 0.f) {
-      fl += pml[i].y * w;
-      float v[DT];
-      part_load<DT>(recv + (i * 8 + fj) * D, fd, v);
-#pragma unroll
-      for (int d = 0; d < DT; ++d) fo[d] += v[d] * w;
-    }
-  }
-  // normalise and write the row's dims (o / l as bf16 hi, lo)
+  // normalise and write the row's positions (o / l as bf16 hi, lo)
   auto write_out = [&](const float* o_, float Ls) {
     write_rows<D, DT>(a, o_, Ls, fr, fd, qt, qn, G, g, r0);
   };
@@ -871,7 +893,7 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
                     make_float2(m[i], l[i]));
       if (m[i] != -INFINITY) {
         const uint32_t dst =
-            ptx::dsmem_map(ptx::smem_u32(recv + (crank * RPC + row) * D + part_pos(0, me.c)), dst_rank);
+            ptx::dsmem_map(ptx::smem_u32(recv + (crank * RPC + row) * D + part_pos(me.c)), dst_rank);
 #pragma unroll
         for (int u = 0; u < DQ / 4; ++u)
           dsmem_st_f4(dst + 64u * u, make_float4(o[i][4 * u], o[i][4 * u + 1], o[i][4 * u + 2], o[i][4 * u + 3]));
@@ -884,7 +906,7 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
     // ---- two chunks in one cluster: CTA r folds rows 4r..4r+3, each
     // chunk's 8 tiles in tile order, then the two chunk partials in chunk
     // order: the arithmetic of the one-chunk fold and of the fold through
-    // memory below (thread: row fj, dims [fd, fd + 4))
+    // memory below (thread: row fj, positions [fd, fd + 4))
     constexpr int TPR = D / 4 < 32 ? D / 4 : 32;  // threads per row
     if (tid < 4 * TPR) {
       const int fj = tid / TPR, fr = 4 * (int)crank + fj, fd = 4 * (tid % TPR);
@@ -892,29 +914,11 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int nh = min(kCluster, n_tiles - (c2 * 2 + h) * kCluster);  // may be <= 0
-        float fm = -INFINITY;
         float2 pml[kCluster];
 #pragma unroll
-        for (int i = 0; i < kCluster; ++i) {
+        for (int i = 0; i < kCluster; ++i)
           pml[i] = (i < nh) ? s_rml[(h * kCluster + i) * 4 + fj] : make_float2(-INFINITY, 0.f);
-          fm = fmaxf(fm, pml[i].x);
-        }
-        float fl = 0.f, fo[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < kCluster; ++i) {
-          const float w = part_weight(pml[i].x, fm);
-          if (w != 0.f) {
-            fl += pml[i].y * w;
-            float v[4];
-            part_load<4>(recv + ((h * kCluster + i) * 4 + fj) * D, fd, v);
-#pragma unroll
-            for (int d = 0; d < 4; ++d) fo[d] += v[d] * w;
-          }
-        }
-        cmx[h] = fm;
-        cls[h] = fl;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) cfo[h][e] = fo[e];
+        fold_tiles<kCluster, 4>(recv + (h * kCluster * 4 + fj) * D + fd, 4 * D, pml, cmx[h], cls[h], cfo[h]);
       }
       if (n_chunks == 1) {
         write_rows<D, 4>(a, cfo[0], cls[0], fr, fd, qt, qn, G, g, r0);
@@ -1163,7 +1167,7 @@ __global__ void __launch_bounds__(128, 4)
                     make_float2(m[i], l[i]));
       if (m[i] != -INFINITY) {
         const uint32_t dst =
-            ptx::dsmem_map(ptx::smem_u32(recv + (rank * 8 + row) * D + part_pos(0, me.c)), dst_rank);
+            ptx::dsmem_map(ptx::smem_u32(recv + (rank * 8 + row) * D + part_pos(me.c)), dst_rank);
 #pragma unroll
         for (int u = 0; u < DQ / 4; ++u)
           dsmem_st_f4(dst + 64u * u, make_float4(o[i][4 * u], o[i][4 * u + 1], o[i][4 * u + 2], o[i][4 * u + 3]));
