@@ -118,6 +118,7 @@ struct AttnArgs {
   int lo_row;
   int32_t* err;
   unsigned long long timeout_ns;
+  int fold_later;         // chunk partials are folded by attn_fold_kernel
   int v_prefetch;         // narrow and quad: bring each tile's V into L2 with its K
   // clusters of request b: [cl_start[b], cl_start[b + 1]); n_ch[b] of them per
   // query tile (chunks covering the host's bound of the request's keys)
@@ -454,9 +455,10 @@ __device__ __forceinline__ void fold_tiles(const float* o, int stride, const flo
 // The fold of a chunk's 8 tile partials for query rows 8 rank .. 8 rank + 7
 // (received into s_rml [8 tiles][8 rows] and recv [8 tiles][8 rows][D]) and
 // what follows it: with one chunk the rows are normalised and written; with
-// several, the rows of the chunk partial go to memory and the last CTA of
-// these rows to arrive folds the chunks in chunk order (9 to stage_max chunks
-// staged in shared memory at sm, whose images are no longer read).
+// several, the rows of the chunk partial go to memory, for attn_fold_kernel
+// (fold_later) or for the last CTA of these rows to arrive, which folds the
+// chunks in chunk order (9 to stage_max chunks staged in shared memory at sm,
+// whose images are no longer read).
 template <int D>
 __device__ __forceinline__ void fold_chunk8(const AttnArgs& a, const float* recv,
                                             const float2* s_rml, int* s_flag, uint8_t* sm,
@@ -495,6 +497,7 @@ __device__ __forceinline__ void fold_chunk8(const AttnArgs& a, const float* recv
       dst[u] = make_float4(fo[4 * u], fo[4 * u + 1], fo[4 * u + 2], fo[4 * u + 3]);
     if ((tid & 15) == 0) a.ws_ml[pc * kQT + fr] = make_float2(fm, fl);
   }
+  if (a.fold_later) return;
   __syncthreads();
   int* cnt = a.cnt + item * kCluster + rank;
   if (tid == 0) {
@@ -954,13 +957,8 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
 // over S, and the second product runs in 64-dim halves of O over S's second
 // half, each read out before the next.  S is read and P written in 16-key
 // chunks, so that no thread holds a whole row of either.
-constexpr uint32_t attn4_smem() { return 32768 + 16384 + 64 * 8 + 8 * 8 + 4 + 16 + 1024; }
+constexpr uint32_t attn4_smem() { return 32768 + 16384 + 64 * 8 + 8 * 8 + 16 + 1024; }
 static_assert(4 * (attn4_smem() + 1024) <= 228 * 1024, "four CTAs per SM");
-// chunks the last arriver stages in shared memory: [11][8 rows][128] floats
-// and [11][8] (max, sum) within the Q and K images
-constexpr int kStage4 = 11;
-static_assert(kStage4 * 8 * 128 * 4 + kStage4 * 8 * 8 <= 32768 + 16384, "staging fits");
-
 template <int D>
 __global__ void __launch_bounds__(128, 4)
     attn_tc4_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -1175,8 +1173,73 @@ __global__ void __launch_bounds__(128, 4)
     }
   }
   ptx::cluster_sync();
-  fold_chunk8<D>(a, recv, s_rml, s_flag, sm, kStage4, rank, c, n_tiles, n_chunks, b, g, qt, qn, G,
-                 r0);
+  fold_chunk8<D>(a, recv, s_rml, s_flag, sm, 0, rank, c, n_tiles, n_chunks, b, g, qt, qn, G, r0);
+}
+
+// The chunk partials of attn_tc4_kernel's requests of several chunks, folded in
+// chunk order (the arithmetic of fold_chunk8's last arriver), normalised and
+// written: one CTA per (query tile, kv head, 8 rows), 16 threads a row, one
+// memory round trip for up to 16 chunks.  With many chunks it costs less than an
+// acquiring arrival at the end of every CTA and a long last one
+// (launch_attention_split has the figures).
+template <int D>
+__global__ void __launch_bounds__(128) attn_fold_kernel(const __grid_constant__ AttnArgs a) {
+  constexpr int DT = D / 16, U = 16;  // positions per thread, chunks in flight
+  const int tid = threadIdx.x, fr = 8 * blockIdx.z + (tid >> 4), fd = DT * (tid & 15);
+  const int G = a.nq / a.nkv, g = blockIdx.y;
+  int b = 0, qt = blockIdx.x;
+  for (;; ++b) {
+    const int tiles = ((a.rm.start[b + 1] - a.rm.start[b]) * G + kQT - 1) / kQT;
+    if (qt < tiles) break;
+    qt -= tiles;
+  }
+  const int r0 = a.rm.start[b], M = a.rm.start[b + 1] - r0, qn = M * G;
+  const size_t pc0 = ((size_t)(b * a.nkv + g) * a.qt_max + qt) * a.chunks_max;
+  const float2* mlp = a.ws_ml + pc0 * kQT + fr;
+  const float* op = a.ws_o + (pc0 * kQT + fr) * D + fd;
+  ptx::griddep_launch_dependents();
+  ptx::griddep_wait();
+  const int L = a.len[b];
+  const int n_tiles = rows_fit(L, M, a.cap) ? (L + M + kTile - 1) / kTile : 0;
+  const int n_chunks = (n_tiles + kCluster - 1) / kCluster;
+  if (n_chunks <= 1 || qt * kQT + fr >= qn) return;
+  float cm = -INFINITY, cl = 0.f, co[DT];
+#pragma unroll
+  for (int i = 0; i < DT; ++i) co[i] = 0.f;
+  for (int c = U; c < n_chunks; ++c) cm = fmaxf(cm, __ldcg(mlp + (size_t)c * kQT).x);
+  for (int c0 = 0; c0 < n_chunks; c0 += U) {
+    float2 ml[U];
+    float4 v[U][DT / 4];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (c0 + u < n_chunks) {
+        ml[u] = __ldcg(mlp + (size_t)(c0 + u) * kQT);
+#pragma unroll
+        for (int i = 0; i < DT / 4; ++i)
+          v[u][i] = __ldcg(reinterpret_cast<const float4*>(op + (size_t)(c0 + u) * kQT * D) + i);
+      }
+    if (c0 == 0) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (u < n_chunks) cm = fmaxf(cm, ml[u].x);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (c0 + u < n_chunks) {
+        const float w = part_weight(ml[u].x, cm);
+        if (w != 0.f) {
+          cl += ml[u].y * w;
+#pragma unroll
+          for (int i = 0; i < DT / 4; ++i) {
+            co[4 * i] += v[u][i].x * w;
+            co[4 * i + 1] += v[u][i].y * w;
+            co[4 * i + 2] += v[u][i].z * w;
+            co[4 * i + 3] += v[u][i].w * w;
+          }
+        }
+      }
+  }
+  write_rows<D, DT>(a, co, cl, fr, fd, qt, qn, G, g, r0);
 }
 
 // Clusters of 16 resident at once, two CTAs per SM: 14 in a residency probe
@@ -1249,26 +1312,15 @@ cudaError_t launch_attn(const CUtensorMap& tk, const CUtensorMap& tv, const Attn
 
 template <int D>
 cudaError_t launch_attn4(const CUtensorMap& tk, const CUtensorMap& tv, const AttnArgs& a,
-                         int clusters, cudaStream_t st) {
+                         int clusters, int q_tiles, bool fold, cudaStream_t st) {
   constexpr uint32_t smem = attn4_smem();
   static const cudaError_t attr = cudaFuncSetAttribute(
       attn_tc4_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (attr != cudaSuccess) return attr;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(clusters * kCluster, a.nkv);
-  cfg.blockDim = dim3(128);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr2[2];
-  attr2[0].id = cudaLaunchAttributeClusterDimension;
-  attr2[0].val.clusterDim.x = kCluster;
-  attr2[0].val.clusterDim.y = 1;
-  attr2[0].val.clusterDim.z = 1;
-  attr2[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr2[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr2;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, attn_tc4_kernel<D>, tk, tv, a);
+  const cudaError_t e = launch_pdl(attn_tc4_kernel<D>, dim3(clusters * kCluster, a.nkv), dim3(128), smem,
+                                   st, kCluster, tk, tv, a);
+  if (e != cudaSuccess || !fold) return e;
+  return launch_pdl(attn_fold_kernel<D>, dim3(q_tiles, a.nkv, kQT / 8), dim3(128), 0, st, 1, a);
 }
 
 }  // namespace
@@ -1341,21 +1393,30 @@ cudaError_t launch_attention_split(const RowMap& m, const Model& md, KvState& kv
     a.cl_start[b + 1] = a.cl_start[b] + attn_q_tiles(m.start[b + 1] - m.start[b], G) *
                                             ((a.n_ch[b] + halves - 1) / halves);
   const int clusters = a.cl_start[kv.batch];
+  // a four-per-SM launch in which a request may have more than four chunks is
+  // followed by the fold of its chunk partials.  Measured, the last arriver's
+  // fold against the kernel, 7B, k = 16: requests of 3500 positions (4 chunks)
+  // 3669 / 3700 us, 5500 (6) 3576 / 3518, 7500 (8) 3423 / 3390, 15128 (15) 3376 /
+  // 3295; 64 requests of the 1.5B of up to two chunks 7213 / 7505.
+  const bool fold = quad && max_nch > 4;
+  a.fold_later = fold ? 1 : 0;
+  int q_tiles = 0;
+  for (int b = 0; b < kv.batch; ++b) q_tiles += attn_q_tiles(m.start[b + 1] - m.start[b], G);
   const dim3 gf(m.rows, (c.n_q_heads + 2 * c.n_kv_heads + kQkvWarps - 1) / kQkvWarps);
   const dim3 bf(32, kQkvWarps);
   cudaError_t e;
-  kv.launches += 2;
+  kv.launches += fold ? 3 : 2;
   if (c.head_dim == 128) {
     e = launch_pdl(qkv_finish_kernel<128>, gf, bf, 0, st, 1, a);
     if (e == cudaSuccess)
-      e = quad     ? launch_attn4<128>(kv.tm_kc, kv.tm_vc, a, clusters, st)
+      e = quad     ? launch_attn4<128>(kv.tm_kc, kv.tm_vc, a, clusters, q_tiles, fold, st)
           : narrow ? launch_attn<128, true, false>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : pair ? launch_attn<128, false, true>(kv.tm_kc, kv.tm_vc, a, clusters, st)
                  : launch_attn<128, false, false>(kv.tm_kc, kv.tm_vc, a, clusters, st);
   } else {
     e = launch_pdl(qkv_finish_kernel<64>, gf, bf, 0, st, 1, a);
     if (e == cudaSuccess)
-      e = quad     ? launch_attn4<64>(kv.tm_kc, kv.tm_vc, a, clusters, st)
+      e = quad     ? launch_attn4<64>(kv.tm_kc, kv.tm_vc, a, clusters, q_tiles, fold, st)
           : narrow ? launch_attn<64, true, false>(kv.tm_kc, kv.tm_vc, a, clusters, st)
           : pair ? launch_attn<64, false, true>(kv.tm_kc, kv.tm_vc, a, clusters, st)
                  : launch_attn<64, false, false>(kv.tm_kc, kv.tm_vc, a, clusters, st);

@@ -59,10 +59,16 @@ def test_rows(pair, rows):
 # tiles; together a launch of four CTAs per SM
 LAYOUT_LENS = [1, 126, 127, 128, 129, 1015, 1023, 1024, 1025, 2030, 2047, 2049, 3000]
 LAYOUT_KS = [0, 1, 16, 0, 3, 9, 0, 16, 2, 16, 0, 8, 12]
+# with requests of more than four chunks: their partials folded by a kernel of
+# their own (17 chunks: two rounds of its loads)
+LONG_LENS = [4080, 4097, 127, 5000, 1024, 6143, 6145, 16500]
+LONG_KS = [16, 0, 9, 16, 3, 1, 16, 12]
 
 
-@pytest.mark.parametrize("d", [64, 128])
-def test_attention_layouts(d):
+@pytest.mark.parametrize("d,lens,ks", [(64, LAYOUT_LENS, LAYOUT_KS), (128, LAYOUT_LENS, LAYOUT_KS),
+                                       (64, LONG_LENS, LONG_KS), (128, LONG_LENS, LONG_KS)],
+                         ids=["d64", "d128", "d64-long", "d128-long"])
+def test_attention_layouts(d, lens, ks):
     """Every request of a large launch equals the same request alone (another
     layout of the attention) bit for bit, and the oracle."""
     import torch
@@ -70,7 +76,7 @@ def test_attention_layouts(d):
         pytest.skip("no GPU")
     cfg = W.ModelConfig(f"d{d}", 1, 256, 8, 2, d, 448, 1032)
     pair = Pair(cfg, seed=0)
-    lens, ks = LAYOUT_LENS * 2, LAYOUT_KS * 2
+    distinct, lens, ks = len(lens), lens * 2, ks * 2
     cap, n = max(lens) + 32, len(lens)
     rng = np.random.default_rng(d)
     roots = [int(x) for x in rng.integers(0, cfg.vocab, size=n)]
@@ -81,7 +87,7 @@ def test_attention_layouts(d):
     kc, vc = st.kc.clone(), st.vc.clone()
     st.close()
     at = 0
-    for b in range(len(LAYOUT_LENS)):
+    for b in range(distinct):
         one = pair.state([lens[b]], cap, [roots[b]])
         one.kc[:, 0, :, :lens[b]] = kc[:, b, :, :lens[b]]
         one.vc[:, 0, :, :lens[b]] = vc[:, b, :, :lens[b]]
