@@ -41,9 +41,15 @@ struct RowMap {
 };
 
 __host__ __device__ inline int row_request(const RowMap& m, int r) {
-  int b = 0;
-  while (b + 1 < m.batch && m.start[b + 1] <= r) ++b;
-  return b;
+  int lo = 0, hi = m.batch - 1;  // the last request that starts at or before row r
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (m.start[mid] <= r)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
 }
 
 // Device error bits (ORed into KvState::d_err); the values of include/as2d.h's

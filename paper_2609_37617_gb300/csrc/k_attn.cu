@@ -10,7 +10,7 @@
 // rows, the second time from L2).
 //
 // qkv_finish_kernel: the QKV projection arrives as split-K partial sums
-// (TC_PART); one warp per (token row, head) adds them in rank order, scales by
+// (TC_PART); half a warp per (token row, head) adds them in rank order, scales by
 // the row's 1 / rms and rotates (RoPE).  Keys and values are appended to the
 // cache; queries, scaled by log2(e) / sqrt(d), are written as bf16 hi and lo
 // parts straight into the tensor-core operand image of their (request, kv
@@ -143,19 +143,22 @@ __device__ __forceinline__ uint32_t img_off(int r, int e) {
 // which a 16-lane TMEM load gives a thread both parts of the same columns.
 __device__ __forceinline__ int hi_row(int q) { return (q >> 3) * 16 + (q & 7); }
 
-// One warp per (token row, head); lane l forms the pairs (e, e + D/2) of e =
-// V l .. V l + V - 1.  Rotate-half RoPE: x' = x cos - x_p sin at e, x_p cos +
+// Half a warp per (token row, head); lane l of it forms the pairs (e, e + D/2)
+// of e = V l .. V l + V - 1.  Rotate-half RoPE: x' = x cos - x_p sin at e, x_p cos +
 // x sin at e + D/2.  Bound by latency, as the residual projections' finishing
 // kernel is (whose comment has the figures of both): addresses before the
-// wait, every load issued before any is used, a warp to a row of a head.  The
+// wait, every load issued before any is used, 16 bytes a lane (D = 128): with a
+// warp to a head and 8 bytes a lane 64 requests of the 1.5B (576 rows) took 6962
+// us, now 6859.  The
 // dependent launch is triggered after the wait: attention CTAs that start
 // before it read the requests' lengths (and measured slower: 7B k = 8 2784 ->
 // 2810 us).
-constexpr int kQkvWarps = 8;  // heads (warps) of one CTA
+constexpr int kQkvWarps = 8;  // warps of one CTA, two heads each
 template <int D>
 __global__ void __launch_bounds__(32 * kQkvWarps) qkv_finish_kernel(const __grid_constant__ AttnArgs a) {
-  constexpr int H2 = D / 2, V = H2 / 32;
-  const int gm = blockIdx.x, head = blockIdx.y * kQkvWarps + threadIdx.y, e = V * threadIdx.x;
+  constexpr int H2 = D / 2, V = H2 / 16;
+  const int gm = blockIdx.x, head = 2 * (blockIdx.y * kQkvWarps + threadIdx.y) + (threadIdx.x >> 4);
+  const int e = V * (threadIdx.x & 15);
   const int b = row_request(a.rm, gm), r0 = a.rm.start[b], i = gm - r0, rows = a.rm.start[b + 1] - r0;
   const bool live = head < a.nq + 2 * a.nkv;
   const bool is_q = head < a.nq, rotate = head < a.nq + a.nkv;
@@ -184,14 +187,16 @@ __global__ void __launch_bounds__(32 * kQkvWarps) qkv_finish_kernel(const __grid
 #pragma unroll
     for (int r = 0; r < 8; ++r)
       if (r < a.qkv_split) {
-        if constexpr (V == 2) {
+        if constexpr (V == 4) {
+          const float4 t0 = __ldcg(reinterpret_cast<const float4*>(s0 + r * part));
+          const float4 t1 = __ldcg(reinterpret_cast<const float4*>(s1 + r * part));
+          v0[r][0] = t0.x, v0[r][1] = t0.y, v0[r][2] = t0.z, v0[r][3] = t0.w;
+          v1[r][0] = t1.x, v1[r][1] = t1.y, v1[r][2] = t1.z, v1[r][3] = t1.w;
+        } else {
           const float2 t0 = __ldcg(reinterpret_cast<const float2*>(s0 + r * part));
           const float2 t1 = __ldcg(reinterpret_cast<const float2*>(s1 + r * part));
           v0[r][0] = t0.x, v0[r][1] = t0.y;
           v1[r][0] = t1.x, v1[r][1] = t1.y;
-        } else {
-          v0[r][0] = __ldcg(s0 + r * part);
-          v1[r][0] = __ldcg(s1 + r * part);
         }
       }
 #pragma unroll
@@ -217,38 +222,38 @@ __global__ void __launch_bounds__(32 * kQkvWarps) qkv_finish_kernel(const __grid
     y0[u] = rotate ? fmaf(x[u], cs[u].x, -(xp[u] * cs[u].y)) : x[u];
     y1[u] = rotate ? fmaf(xp[u], cs[u].x, x[u] * cs[u].y) : xp[u];
   }
-  // V consecutive bf16 (4-byte aligned for V = 2)
-  auto put = [](void* to, const bf16* v) {
-    if constexpr (V == 2)
-      *reinterpret_cast<__nv_bfloat162*>(to) = __halves2bfloat162(v[0], v[1]);
+  // V consecutive bf16 (8- or 4-byte aligned)
+  auto put = [](void* to, const float* v) {
+    uint32_t w[V / 2];
+#pragma unroll
+    for (int u = 0; u < V / 2; ++u) {
+      const __nv_bfloat162 t = __floats2bfloat162_rn(v[2 * u], v[2 * u + 1]);
+      w[u] = *reinterpret_cast<const uint32_t*>(&t);
+    }
+    if constexpr (V == 4)
+      *reinterpret_cast<uint2*>(to) = make_uint2(w[0], w[1]);
     else
-      *reinterpret_cast<bf16*>(to) = v[0];
+      *reinterpret_cast<uint32_t*>(to) = w[0];
   };
   if (is_q) {
-    bf16 h0[V], h1[V], l0[V], l1[V];
+    // hi parts, and what they leave (exact) as lo parts
+    float l0[V], l1[V];
 #pragma unroll
     for (int u = 0; u < V; ++u) {
-      const float w0 = y0[u] * a.qscale, w1 = y1[u] * a.qscale;
-      h0[u] = __float2bfloat16_rn(w0);
-      h1[u] = __float2bfloat16_rn(w1);
-      l0[u] = __float2bfloat16_rn(w0 - __bfloat162float(h0[u]));
-      l1[u] = __float2bfloat16_rn(w1 - __bfloat162float(h1[u]));
+      y0[u] *= a.qscale;
+      y1[u] *= a.qscale;
+      l0[u] = y0[u] - __bfloat162float(__float2bfloat16_rn(y0[u]));
+      l1[u] = y1[u] - __bfloat162float(__float2bfloat16_rn(y1[u]));
     }
     const int row = hi_row(q);
-    put(img + img_off(row, e), h0);
-    put(img + img_off(row, e + H2), h1);
+    put(img + img_off(row, e), y0);
+    put(img + img_off(row, e + H2), y1);
     put(img + img_off(row + 8, e), l0);
     put(img + img_off(row + 8, e + H2), l1);
   } else {
-    bf16 k0[V], k1[V];
-#pragma unroll
-    for (int u = 0; u < V; ++u) {
-      k0[u] = __float2bfloat16_rn(y0[u]);
-      k1[u] = __float2bfloat16_rn(y1[u]);
-    }
     dst += (size_t)(len_b + i) * D;
-    put(dst, k0);
-    put(dst + H2, k1);
+    put(dst, y0);
+    put(dst + H2, y1);
   }
 }
 
@@ -1402,7 +1407,7 @@ cudaError_t launch_attention_split(const RowMap& m, const Model& md, KvState& kv
   a.fold_later = fold ? 1 : 0;
   int q_tiles = 0;
   for (int b = 0; b < kv.batch; ++b) q_tiles += attn_q_tiles(m.start[b + 1] - m.start[b], G);
-  const dim3 gf(m.rows, (c.n_q_heads + 2 * c.n_kv_heads + kQkvWarps - 1) / kQkvWarps);
+  const dim3 gf(m.rows, (c.n_q_heads + 2 * c.n_kv_heads + 2 * kQkvWarps - 1) / (2 * kQkvWarps));
   const dim3 bf(32, kQkvWarps);
   cudaError_t e;
   kv.launches += fold ? 3 : 2;
