@@ -28,6 +28,24 @@ def pair():
                                   [17] * 8, [17] * 10, [17] * 12, [16] * 16, [17] * 15 + [2], [17] * 16],
                          ids=lambda r: f"{sum(r)}rows")
 def test_rows(pair, rows):
+    check_rows(pair, rows)
+
+
+# Few SMs give each CTA enough units for pairs of CTAs: with 2, whole tiles of
+# odd counts (gate/up 23, down 3, vocabulary 9), with 4 also tiles of the
+# residual projections cut between CTAs.  NB = 64, 96, 192, 256 and 16.
+@pytest.mark.parametrize("sms", [2, 4])
+@pytest.mark.parametrize("rows", [[16] * 4, [17] * 4, [17] * 10, [17] * 16], ids=lambda r: f"{sum(r)}rows")
+def test_rows_few_sms(rows, sms):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    few = Pair(W.ModelConfig("odd-few", 2, 384, 6, 2, 64, 1472, 1032), seed=0, gains="random")
+    few.model.set_sm_budget(sms)
+    check_rows(few, rows)
+
+
+def check_rows(pair, rows):
     cfg, n = pair.cfg, len(rows)
     rng = np.random.default_rng(sum(rows))
     lens = [int(x) for x in rng.integers(1, CAP - 20, size=n)]
