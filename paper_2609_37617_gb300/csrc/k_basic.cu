@@ -45,27 +45,26 @@ __global__ void __launch_bounds__(128) embed_kernel(
   const int r = blockIdx.x;
   const int b = row_request(m, r);
   const int i = r - m.start[b];
+  // the token and the length first: the table row's load waits for the token,
+  // and nothing may stand between them
+  int tok = (i == 0) ? (root_override ? root_override[b] : root[b]) : cand[m.start[b] - b + i - 1];
+  const int L = len[b];
+  const bool bad_tok = tok < 0 || tok >= V;
   // a request whose length leaves no room for its rows is flagged and skipped
   // downstream (rows_fit); its rows take position 0's rotary entries
-  const bool fits = rows_fit(len[b], m.start[b + 1] - m.start[b], cap);
-  if (!fits && threadIdx.x == 0) {
-    atomicOr(err, kErrCapacity);
+  const bool fits = rows_fit(L, m.start[b + 1] - m.start[b], cap);
+  float2 cs = make_float2(0.f, 0.f);
+  if ((int)threadIdx.x < d / 2) {
+    const int e = threadIdx.x, pos = fits ? L + i : 0;
+    cs = rope_full ? rope_full[(size_t)pos * (d / 2) + e] : rope_angle(pos, e, d, theta);
+  }
+  if (bad_tok) tok = 0;
+  embed_row_body(E + (size_t)tok * H, g0, H, r, ss_ld, h, xn, ss, threadIdx.x, 128, part, 0);
+  if ((int)threadIdx.x < d / 2) rope[(size_t)r * (d / 2) + threadIdx.x] = cs;
+  if (threadIdx.x == 0 && (!fits || bad_tok)) {
+    atomicOr(err, (fits ? 0 : kErrCapacity) | (bad_tok ? kErrBadToken : 0));
     bad[b] = 1;
   }
-  if ((int)threadIdx.x < d / 2) {
-    const int e = threadIdx.x, pos = fits ? len[b] + i : 0;
-    rope[(size_t)r * (d / 2) + e] =
-        rope_full ? rope_full[(size_t)pos * (d / 2) + e] : rope_angle(pos, e, d, theta);
-  }
-  int tok = (i == 0) ? (root_override ? root_override[b] : root[b]) : cand[m.start[b] - b + i - 1];
-  if (tok < 0 || tok >= V) {
-    if (threadIdx.x == 0) {
-      atomicOr(err, kErrBadToken);
-      bad[b] = 1;
-    }
-    tok = 0;
-  }
-  embed_row_body(E + (size_t)tok * H, g0, H, r, ss_ld, h, xn, ss, threadIdx.x, 128, part, 0);
 }
 
 // ---- accept scan + state update ---------------------------------------------------

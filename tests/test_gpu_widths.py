@@ -45,6 +45,16 @@ def test_rows_few_sms(rows, sms):
     check_rows(few, rows)
 
 
+# The embedding's 14 columns a thread in one batch (1792) and one more (1920).
+@pytest.mark.parametrize("hidden", [1792, 1920])
+def test_rows_embed_batches(hidden):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    check_rows(Pair(W.ModelConfig("odd-embed", 1, hidden, hidden // 64, 2, 64, 448, 1032), seed=0, gains="random"),
+               [4, 1, 3])
+
+
 def check_rows(pair, rows):
     cfg, n = pair.cfg, len(rows)
     rng = np.random.default_rng(sum(rows))
