@@ -415,10 +415,12 @@ extern "C" void as2d_kv_free(as2d_kv* kh) {
   cudaFree(kh->s.rope_full);
   cudaFree(kh->s.cb_dev);
   cudaFree(kh->s.pf_out);
-  if (kh->s.pf) {
-    // the prefill state's lengths, roots, flags and rotary table are this state's
-    cudaFree(kh->s.pf->work);
-    delete kh->s.pf;
+  for (KvState* w = kh->s.pf; w;) {
+    // the prefill states' lengths, roots, flags and rotary table are this state's
+    KvState* next = w->pf;
+    cudaFree(w->work);
+    delete w;
+    w = next;
   }
   cudaFreeHost(kh->s.cb_host);
   delete kh;
@@ -611,6 +613,43 @@ as2d_status run_block(KvState& s, const int32_t* cand, const int32_t* k,
 
 }  // namespace
 
+namespace {
+
+// A prefill working state of `rows` rows a pass, zeroed in the stream's order
+// and put before the ones that s has: those stay until as2d_kv_free, as a
+// captured graph may hold their addresses (at most one of each of 64, 128 and
+// 256 rows).
+as2d_status make_prefill_state(KvState& s, int rows, cudaStream_t st) {
+  KvState* a = new KvState();
+  a->model = s.model;
+  a->batch = 1;
+  a->capacity = s.capacity;
+  a->k_cache = s.k_cache;
+  a->v_cache = s.v_cache;
+  a->len_upper = s.len_upper;
+  as2d_status rc = alloc_work(*a, *s.model, 1, s.capacity, rows);
+  if (rc == AS2D_OK) {
+    const cudaError_t e = cudaMemsetAsync(a->work, 0, a->work_bytes, st);
+    if (e != cudaSuccess) {
+      cudaFree(a->work);
+      rc = fail(AS2D_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+    }
+  }
+  if (rc != AS2D_OK) {
+    delete a;
+    return rc;
+  }
+  a->d_len = s.d_len;
+  a->d_root = s.d_root;
+  a->d_err = s.d_err;
+  a->rope_full = s.rope_full;
+  a->pf = s.pf;
+  s.pf = a;
+  return AS2D_OK;
+}
+
+}  // namespace
+
 extern "C" as2d_status as2d_prefill(as2d_kv* kh, const int32_t* tokens, int32_t n,
                                     int32_t* first_token, void* stream) {
   g_err.clear();
@@ -627,48 +666,28 @@ extern "C" as2d_status as2d_prefill(as2d_kv* kh, const int32_t* tokens, int32_t 
     }
   }
   // The working state of the passes.  A call longer than the state was made
-  // for makes a larger one in its place, unless that cannot be had (a stream
-  // under capture, no memory): its passes are then of the size there is.
+  // for makes a larger one, unless that cannot be had (a stream under capture,
+  // no memory): its passes are then of the size there is, or of the smallest.
   const int want = prefill_rows(n);
-  bool make = !s.pf;
-  if (s.pf && want > s.pf->max_rows) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    make = cudaStreamIsCapturing((cudaStream_t)stream, &cap) == cudaSuccess &&
-           cap == cudaStreamCaptureStatusNone;
-    if (!make) (void)cudaGetLastError();
-  }
-  if (make) {
-    KvState* a = new KvState();
-    a->model = s.model;
-    a->batch = 1;
-    a->capacity = s.capacity;
-    a->k_cache = s.k_cache;
-    a->v_cache = s.v_cache;
-    a->len_upper = s.len_upper;
-    as2d_status rc = alloc_work(*a, *s.model, 1, s.capacity, want);
-    if (rc == AS2D_OK) {
-      const cudaError_t e = cudaMemset(a->work, 0, a->work_bytes);
-      if (e != cudaSuccess) {
-        cudaFree(a->work);
-        rc = fail(AS2D_ERR_CUDA, std::string("cudaMemset: ") + cudaGetErrorString(e));
-      }
-    }
-    if (rc != AS2D_OK) {
-      delete a;
-      if (!s.pf) return rc;
+  if (!s.pf) {
+    as2d_status rc = make_prefill_state(s, want, (cudaStream_t)stream);
+    if (rc != AS2D_OK && want > prefill_rows(1)) {
       (void)cudaGetLastError();
       g_err.clear();
-    } else {
-      a->d_len = s.d_len;
-      a->d_root = s.d_root;
-      a->d_err = s.d_err;
-      a->rope_full = s.rope_full;
-      if (s.pf) {
-        cudaFree(s.pf->work);  // waits for the calls that still use it
-        delete s.pf;
-      }
-      s.pf = a;
+      rc = make_prefill_state(s, prefill_rows(1), (cudaStream_t)stream);
     }
+    if (rc != AS2D_OK) return rc;
+  } else if (want > s.pf->max_rows) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) == cudaSuccess &&
+        cap == cudaStreamCaptureStatusNone) {
+      // a capture on another thread must not be ended by this allocation
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+      if (make_prefill_state(s, want, (cudaStream_t)stream) != AS2D_OK) g_err.clear();
+      if (swapped) (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    (void)cudaGetLastError();
   }
   KvState& w = *s.pf;
   w.len_upper = s.len_upper;

@@ -240,8 +240,9 @@ struct KvState {
   int32_t* cb_host = nullptr;            // pinned, same layout
   int32_t* pf_out = nullptr;             // [2] n_accepted, root of as2d_prefill chunks
   // as2d_prefill's working state (batch 1, prefill_rows(n) rows per pass), made
-  // on first use and again for a longer call; shares this state's cache,
-  // lengths, roots, error flags and rotary table
+  // on first use and a larger one for a longer call, the smaller behind it in
+  // its own pf; shares this state's cache, lengths, roots, error flags and
+  // rotary table
   KvState* pf = nullptr;
 };
 

@@ -118,6 +118,43 @@ def test_prefill_wide_passes(pair, n, chunks):
     ref.close()
 
 
+def test_prefill_graph_outlives_growth(pair):
+    """A prefill captured into a graph replays after a longer call has made a
+    larger working state, and a long call under capture takes the passes of
+    the state there is."""
+    import torch
+    cfg, n = pair.cfg, 200
+    instr = torch_tokens(cfg, n + 8)
+    ref = pair.state([L0], L0 + 512, [0])
+    first_ref = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref.prefill(instr[:8], first_ref)
+    ref.prefill(instr[8:8 + n], first_ref)
+
+    st = pair.state([L0], L0 + 512, [0])
+    first = torch.zeros(1, dtype=torch.int32, device="cuda")
+    st.prefill(instr[:8], first)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        st.prefill(instr[8:8 + n], first, stream=side.cuda_stream)
+    torch.cuda.synchronize()
+    st.rollback([L0], [0])
+    st.prefill(instr[:n], first)  # eager: makes the larger state
+    st.rollback([L0 + 8], [0])
+    graph.replay()
+    torch.cuda.synchronize()
+    st.check()
+    assert int(first.item()) == int(first_ref.item())
+    assert st.read_state() == ref.read_state()
+    for l in range(cfg.n_layers):
+        for a, b in ((st.kc, ref.kc), (st.vc, ref.vc)):
+            assert np.array_equal(bf16_bits(a[l, 0])[:, :L0 + 8 + n], bf16_bits(b[l, 0])[:, :L0 + 8 + n])
+    st.close()
+    ref.close()
+
+
 def torch_tokens(cfg, n):
     import torch
     return torch.tensor([int(t) for t in W.instruction_tokens(cfg, n, 2)], dtype=torch.int32, device="cuda")
