@@ -698,8 +698,14 @@ extern "C" as2d_status as2d_prefill(as2d_kv* kh, const int32_t* tokens, int32_t 
   // row of every pass it was 0.4 of the 7.4 ms of 300 tokens of the 1.5B.
   const int pass = w.max_rows < want ? w.max_rows : want;
   as2d_status rc = AS2D_OK;
-  for (int s0 = 0; s0 < n && rc == AS2D_OK; s0 += pass) {
-    const int rows = (n - s0) < pass ? (n - s0) : pass;
+  for (int s0 = 0, rows = 0; s0 < n && rc == AS2D_OK; s0 += rows) {
+    const int left = n - s0;
+    rows = left < pass ? left : pass;
+    // a full pass and up to 64 rows cost more than two passes of up to 160
+    // (256 + r against halves, us: 1.5B with r = 1 / 44 / 74 / 134 3464 / 3659
+    // / 3784 / 4207 against 3313 / 3576 / 3702 / 4388, 7B with r = 1 / 44 / 144
+    // 8624 / 8984 / 10509 against 7904 / 8620 / 10700)
+    if (pass == kPrefillMaxRows && left > pass && left <= pass + 64) rows = (left + 1) / 2;
     const int32_t k = rows - 1;
     const bool last = s0 + rows == n;
     const as2d_verify_out out{s.pf_out, (last && first_token) ? first_token : s.pf_out + 1,

@@ -87,11 +87,12 @@ def test_prefill_is_chunking_invariant(pair, chunks):
     ref.close()
 
 
-@pytest.mark.parametrize("n,chunks", [(256, [64, 64, 128]), (257, [64, 193]), (300, [129, 171])])
+@pytest.mark.parametrize("n,chunks", [(256, [64, 64, 128]), (257, [64, 193]), (300, [129, 171]), (320, [257, 63]), (321, [321]),
+                                      (513, [200, 313])])
 def test_prefill_wide_passes(pair, n, chunks):
-    """Passes of up to 256 rows, one row past a pass, and calls that outgrow
-    the working state of the call before them (64 -> 128 -> 256 rows): bitwise
-    the cache and first token of one call."""
+    """Passes of up to 256 rows; 1, 44 and 64 rows past a pass (two halves) and
+    65; and calls that outgrow the working state of the call before them (64 ->
+    128 -> 256 rows): bitwise the cache and first token of one call."""
     cfg, cap = pair.cfg, L0 + n + 4
     instr = torch_tokens(cfg, n)
 
