@@ -527,9 +527,14 @@ cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, co
   p.err = s.d_err;
   p.timeout_ns = s.wait_ns;
   p.rm = rm;
-  for (int row0 = first_row; row0 < rm.rows; row0 += 256) {
+  for (int row0 = first_row; row0 < rm.rows; row0 += p.rows) {
+    // launches of 256 rows; what is at most 64 over goes in two halves (whole
+    // passes, us, 256 + r against halves: 272 / 306 / 320 rows of the 1.5B
+    // 3324 / 3509 / 3594 against 3298 / 3434 / 3517, of the 7B 8467 / 8700 /
+    // 8840 against 8245 / 8440 / 8560, 576 of the 1.5B 6630 against 6608)
+    const int left = rm.rows - row0;
     p.row0 = row0;
-    p.rows = rm.rows - row0 < 256 ? rm.rows - row0 : 256;
+    p.rows = left <= 256 ? left : left <= 320 ? (left + 1) / 2 : 256;
     const int nb = nb_for_rows(p.rows), i = nb_index(nb);
     const TcMaps maps{&x.maps[i], &x.pair[i], &wmap};
     cudaError_t e;
