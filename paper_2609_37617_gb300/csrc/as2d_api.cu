@@ -479,6 +479,19 @@ struct Operand {
   const CUtensorMap *maps, *pair;  // per token-row padding
 };
 
+// Rows of a projection's next launch, of `left`: equal shares where they pad
+// to 160 or 192 rows, else 256 first.  Whole passes, us, 256 first against
+// shares: 272 / 306 / 320 / 384 rows of the 1.5B 3324 / 3509 / 3594 / 3909
+// against 3298 / 3434 / 3517 / 3798, of the 7B 8467 / 8700 / 8840 / 9713
+// against 8245 / 8440 / 8560 / 9580; 576 rows as 3 x 192 against 256 + 160 +
+// 160 6404 / 6572 and 14460 / 14945; 256 + 96 is the better of 2 x 176 (352
+// rows 3700 / 3709 and 9370 / 9470), and 256 + 134 of 2 x 195.
+int launch_rows(int left) {
+  const int n = (left + 255) / 256, share = (left + n - 1) / n;
+  if (n == 1) return left;
+  return share <= 160 || (share <= 192 && left > 352) ? share : 256;
+}
+
 cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, const bf16* w,
                        const CUtensorMap& wmap, const Operand& x, int N, int K, TcParams p,
                        cudaStream_t st, int first_row = 0) {
@@ -528,13 +541,8 @@ cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, co
   p.timeout_ns = s.wait_ns;
   p.rm = rm;
   for (int row0 = first_row; row0 < rm.rows; row0 += p.rows) {
-    // launches of 256 rows; what is at most 64 over goes in two halves (whole
-    // passes, us, 256 + r against halves: 272 / 306 / 320 rows of the 1.5B
-    // 3324 / 3509 / 3594 against 3298 / 3434 / 3517, of the 7B 8467 / 8700 /
-    // 8840 against 8245 / 8440 / 8560, 576 of the 1.5B 6630 against 6608)
-    const int left = rm.rows - row0;
     p.row0 = row0;
-    p.rows = left <= 256 ? left : left <= 320 ? (left + 1) / 2 : 256;
+    p.rows = launch_rows(rm.rows - row0);
     const int nb = nb_for_rows(p.rows), i = nb_index(nb);
     const TcMaps maps{&x.maps[i], &x.pair[i], &wmap};
     cudaError_t e;
