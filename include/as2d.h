@@ -165,9 +165,10 @@ as2d_status as2d_verify_block(as2d_kv* kv, const int32_t* candidates,
    L .. L + n - 1 of a batch-1 state and keeps every entry, in passes of up
    to 256 rows through the verification pass (the first call allocates a
    working state for passes of 64, 128 or 256 rows, whichever holds its n, and
-   a longer call a larger one, all kept until as2d_kv_free; under stream
+   a longer call a larger one, all kept until as2d_kv_free.  Under stream
    capture, or without the memory, a call uses the one there is, in more
-   passes, or on first use one of 64 rows.  Its attention
+   passes, or on first use makes one of 64 rows; that state is ready when the
+   call returns, whether or not the captured graph ever runs.  Its attention
    buffers grow with the capacity, by about 3.7 MB per 1024 positions for the
    7B shape and 256 rows).  The LM head runs over the last row only.  The pending root
    before the call is discarded; afterwards L' = L + n and the root is the

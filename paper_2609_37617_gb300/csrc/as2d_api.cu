@@ -628,11 +628,34 @@ as2d_status run_block(KvState& s, const int32_t* cand, const int32_t* k,
 
 namespace {
 
-// A prefill working state of `rows` rows a pass, zeroed in the stream's order
-// and put before the ones that s has: those stay until as2d_kv_free, as a
-// captured graph may hold their addresses (at most one of each of 64, 128 and
-// 256 rows).
-as2d_status make_prefill_state(KvState& s, int rows, cudaStream_t st) {
+// While one of these lives, this thread may allocate beside a stream capture,
+// its own or another thread's, which goes on undisturbed.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+  ~RelaxedCapture() {
+    if (swapped) (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+};
+
+// Zeroes fresh device memory before it returns, on a stream of its own: on the
+// caller's the memset of a call under capture would only become a node of the
+// graph, and calls that run before that graph does (or without it, if it is
+// dropped) would find what the allocation held.
+cudaError_t zero_now(void* p, size_t bytes) {
+  cudaStream_t st = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p, 0, bytes, st);
+  const cudaError_t done = cudaStreamSynchronize(st);
+  (void)cudaStreamDestroy(st);
+  return e != cudaSuccess ? e : done;
+}
+
+// A prefill working state of `rows` rows a pass, put before the ones that s
+// has: those stay until as2d_kv_free, as a captured graph may hold their
+// addresses (at most one of each of 64, 128 and 256 rows).
+as2d_status make_prefill_state(KvState& s, int rows) {
   KvState* a = new KvState();
   a->model = s.model;
   a->batch = 1;
@@ -642,10 +665,10 @@ as2d_status make_prefill_state(KvState& s, int rows, cudaStream_t st) {
   a->len_upper = s.len_upper;
   as2d_status rc = alloc_work(*a, *s.model, 1, s.capacity, rows);
   if (rc == AS2D_OK) {
-    const cudaError_t e = cudaMemsetAsync(a->work, 0, a->work_bytes, st);
+    const cudaError_t e = zero_now(a->work, a->work_bytes);
     if (e != cudaSuccess) {
       cudaFree(a->work);
-      rc = fail(AS2D_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+      rc = fail(AS2D_ERR_CUDA, std::string("zeroing the working memory: ") + cudaGetErrorString(e));
     }
   }
   if (rc != AS2D_OK) {
@@ -661,6 +684,36 @@ as2d_status make_prefill_state(KvState& s, int rows, cudaStream_t st) {
   return AS2D_OK;
 }
 
+// What a prefill of `want` rows a pass needs.  A call longer than the state
+// was made for makes a larger one, unless that cannot be had (a stream under
+// capture, no memory): its passes are then of the size there is, on first use
+// of 64 rows.
+as2d_status ensure_prefill_state(KvState& s, int want, cudaStream_t st) {
+  if (s.pf_out && s.pf && want <= s.pf->max_rows) return AS2D_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool captured =
+      cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  const RelaxedCapture relaxed;
+  if (!s.pf_out) {
+    const cudaError_t e = cudaMalloc(&s.pf_out, 2 * sizeof(int32_t));
+    if (e != cudaSuccess) {
+      s.pf_out = nullptr;
+      return fail(AS2D_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
+  }
+  const int least = prefill_rows(1);
+  as2d_status rc = AS2D_OK;
+  if (!s.pf && captured)
+    rc = make_prefill_state(s, least);
+  else if (!captured && (!s.pf || want > s.pf->max_rows))
+    rc = make_prefill_state(s, want);
+  if (rc != AS2D_OK && !s.pf && !captured && want > least) rc = make_prefill_state(s, least);
+  (void)cudaGetLastError();
+  if (!s.pf) return rc;
+  g_err.clear();
+  return AS2D_OK;
+}
+
 }  // namespace
 
 extern "C" as2d_status as2d_prefill(as2d_kv* kh, const int32_t* tokens, int32_t n,
@@ -671,37 +724,9 @@ extern "C" as2d_status as2d_prefill(as2d_kv* kh, const int32_t* tokens, int32_t 
   if (s.batch != 1) return fail(AS2D_ERR_UNSUPPORTED, "prefill runs batch-1 states");
   if (s.len_upper[0] + n > s.capacity)
     return fail(AS2D_ERR_CAPACITY, "length bound + n exceeds the cache capacity");
-  if (!s.pf_out) {
-    const cudaError_t e = cudaMalloc(&s.pf_out, 2 * sizeof(int32_t));
-    if (e != cudaSuccess) {
-      s.pf_out = nullptr;
-      return fail(AS2D_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    }
-  }
-  // The working state of the passes.  A call longer than the state was made
-  // for makes a larger one, unless that cannot be had (a stream under capture,
-  // no memory): its passes are then of the size there is, or of the smallest.
   const int want = prefill_rows(n);
-  if (!s.pf) {
-    as2d_status rc = make_prefill_state(s, want, (cudaStream_t)stream);
-    if (rc != AS2D_OK && want > prefill_rows(1)) {
-      (void)cudaGetLastError();
-      g_err.clear();
-      rc = make_prefill_state(s, prefill_rows(1), (cudaStream_t)stream);
-    }
-    if (rc != AS2D_OK) return rc;
-  } else if (want > s.pf->max_rows) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) == cudaSuccess &&
-        cap == cudaStreamCaptureStatusNone) {
-      // a capture on another thread must not be ended by this allocation
-      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-      const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
-      if (make_prefill_state(s, want, (cudaStream_t)stream) != AS2D_OK) g_err.clear();
-      if (swapped) (void)cudaThreadExchangeStreamCaptureMode(&mode);
-    }
-    (void)cudaGetLastError();
-  }
+  const as2d_status ready = ensure_prefill_state(s, want, (cudaStream_t)stream);
+  if (ready != AS2D_OK) return ready;
   KvState& w = *s.pf;
   w.len_upper = s.len_upper;
   w.wait_ns = s.wait_ns;

@@ -2,6 +2,8 @@
 workload's 150 retained "audio" positions plus 50 instruction tokens
 prefilled by the library, against the oracle; chunking invariance; the
 first verification block after it; argument errors."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -154,6 +156,65 @@ def test_prefill_graph_outlives_growth(pair):
             assert np.array_equal(bf16_bits(a[l, 0])[:, :L0 + 8 + n], bf16_bits(b[l, 0])[:, :L0 + 8 + n])
     st.close()
     ref.close()
+
+
+@pytest.mark.parametrize("mode", ["relaxed", "thread_local", "global"])
+def test_first_prefill_under_capture(pair, mode):
+    """The first prefill of a state, captured: the graph holds kernels alone, so
+    the working state does not wait for a replay to be cleared, and calls before
+    the first replay, replays and calls after it give bitwise what a fresh state
+    gives."""
+    import torch
+    cfg, n = pair.cfg, 100
+    instr = torch_tokens(cfg, n)
+    ref = pair.state([L0], L0 + 256, [0])
+    first_ref = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref.prefill(instr, first_ref)
+    torch.cuda.synchronize()
+
+    st = pair.state([L0], L0 + 256, [0])
+    first = torch.zeros(1, dtype=torch.int32, device="cuda")
+    side = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=side, capture_error_mode=mode):
+        st.prefill(instr, first, stream=side.cuda_stream)
+    assert set(graph_node_types(graph.raw_cuda_graph())) == {0}  # cudaGraphNodeTypeKernel
+
+    def check():
+        torch.cuda.synchronize()
+        st.check()
+        assert int(first.item()) == int(first_ref.item())
+        assert st.read_state() == ref.read_state()
+        for l in range(cfg.n_layers):
+            for a, b in ((st.kc, ref.kc), (st.vc, ref.vc)):
+                assert np.array_equal(bf16_bits(a[l, 0])[:, :L0 + n], bf16_bits(b[l, 0])[:, :L0 + n])
+        first.fill_(-7)
+        st.rollback([L0], [0])
+
+    st.rollback([L0], [0])  # (the captured call raised the host's bound of the length)
+    st.prefill(instr[:64], first)  # the state that the captured call made, before any replay
+    st.prefill(instr[64:], first)
+    check()
+    graph.replay()
+    check()
+    st.prefill(instr, first)
+    check()
+    st.close()
+    ref.close()
+
+
+def graph_node_types(graph):
+    """cudaGraphNodeType of every node of a cudaGraph_t."""
+    rt = ctypes.CDLL("libcudart.so.13")
+    n = ctypes.c_size_t(0)
+    assert rt.cudaGraphGetNodes(ctypes.c_void_p(graph), None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert rt.cudaGraphGetNodes(ctypes.c_void_p(graph), nodes, ctypes.byref(n)) == 0
+    kind, kinds = ctypes.c_int(), []
+    for node in nodes:
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    return kinds
 
 
 def torch_tokens(cfg, n):
