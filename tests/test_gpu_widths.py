@@ -47,6 +47,49 @@ def test_rows_few_sms(rows, sms):
     check_rows(few, rows)
 
 
+def check_wait_limits(pair, lens, cap, ks):
+    """Calls whose kernels' waits run out, at once or somewhere on the way (the
+    limits, ns), report it, and leave a state that gives the same bits again."""
+    import paper_2609_37617_gb300 as lib
+    rng = np.random.default_rng(len(lens))
+    roots = [int(x) for x in rng.integers(0, pair.cfg.vocab, size=len(lens))]
+    cands = [[int(t) for t in rng.integers(0, pair.cfg.vocab, size=k)] for k in ks]
+    st = pair.state(lens, cap, roots)
+    want = run_gpu_block(st, pair.cfg, cands)
+    st.check()
+    st.rollback(lens, roots)
+    for limit in (0, 500, 1000, 2000, 4000, 8000, 16000, 32000):
+        st.set_wait_limit(limit)
+        for _ in range(4):
+            run_gpu_block(st, pair.cfg, cands, want_logits=False)
+            st.rollback(lens, roots)
+        try:
+            st.check()
+            assert limit > 0, "a limit of 0 runs out"
+        except lib.AS2DError as e:
+            assert e.status == lib.AS2D_ERR_DEVICE and "timed out" in str(e)
+        st.set_wait_limit(2_000_000_000)
+        st.rollback(lens, roots)
+        for a, b in zip(run_gpu_block(st, pair.cfg, cands), want):
+            assert np.array_equal(a, b)
+        st.check()
+        st.rollback(lens, roots)
+    st.close()
+
+
+# pairs of CTAs with one accumulator and with two, whole and split tiles
+@pytest.mark.parametrize("sms", [2, 4, 32])
+@pytest.mark.parametrize("rows", [[16] * 4, [17] * 6, [17] * 10, [17] * 16], ids=lambda r: f"{sum(r)}rows")
+def test_wait_limits_pairs(rows, sms):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    few = Pair(W.ModelConfig("odd-few", 2, 384, 6, 2, 64, 1472, 1032), seed=0, gains="random")
+    few.model.set_sm_budget(sms)
+    check_wait_limits(few, [int(x) for x in np.random.default_rng(0).integers(1, CAP - 20, size=len(rows))], CAP,
+                      [r - 1 for r in rows])
+
+
 # The embedding's 14 columns a thread in one batch (1792) and one more (1920).
 @pytest.mark.parametrize("hidden", [1792, 1920])
 def test_rows_embed_batches(hidden):
@@ -127,3 +170,14 @@ def test_attention_layouts(d, lens, ks):
         want = pair.oracle.verify_block(pair.oracle_cache(lens[b], cap, req=b), lens[b], roots[b], cands[b])
         assert np.max(np.abs(want["logits"] - rows)) <= LOGIT_TOL, f"length {lens[b]}"
         at += ks[b] + 1
+
+
+# three CTAs per SM (17 requests of a chunk: 34 clusters), four, four with the fold kernel
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lens", [[1015] * 17, LAYOUT_LENS * 2, LONG_LENS], ids=["three", "four", "fold"])
+def test_wait_limits_attention(d, lens):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    check_wait_limits(Pair(W.ModelConfig(f"d{d}", 1, 256, 8, 2, d, 448, 1032), seed=0), lens, max(lens) + 32,
+                      [3 + i % 5 for i in range(len(lens))])
