@@ -825,11 +825,14 @@ extern "C" as2d_status as2d_kv_check(as2d_kv* kh, void* stream) {
   if (err != 0) {
     int32_t zero = 0;
     CUDA_TRY(cudaMemcpy(kh->s.d_err, &zero, 4, cudaMemcpyHostToDevice));
-    // a kernel that gave up may have left split-tile arrival counts behind
-    if (kh->s.counters && kh->s.n_counters > 0)
-      CUDA_TRY(cudaMemset(kh->s.counters, 0, (size_t)kh->s.n_counters * 4));
-    if (kh->s.attn_cnt && kh->s.n_attn_cnt > 0)
-      CUDA_TRY(cudaMemset(kh->s.attn_cnt, 0, (size_t)kh->s.n_attn_cnt * 4));
+    // a kernel that gave up may have left split-tile arrival counts behind, in
+    // this state's working memory or in its prefill passes'
+    for (const KvState* w = &kh->s; w; w = w->pf) {
+      if (w->counters && w->n_counters > 0)
+        CUDA_TRY(cudaMemset(w->counters, 0, (size_t)w->n_counters * 4));
+      if (w->attn_cnt && w->n_attn_cnt > 0)
+        CUDA_TRY(cudaMemset(w->attn_cnt, 0, (size_t)w->n_attn_cnt * 4));
+    }
     std::string msg = "device error:";
     if (err & kErrBadToken) msg += " candidate or root token outside [0, vocab);";
     if (err & kErrRollback) msg += " rollback beyond the committed length;";

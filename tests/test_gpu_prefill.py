@@ -203,6 +203,41 @@ def test_first_prefill_under_capture(pair, mode):
     ref.close()
 
 
+@pytest.mark.parametrize("n", [40, 100, 300])
+def test_prefill_recovers_from_expired_waits(pair, n):
+    """A prefill whose kernels' waits run out reports it; the next one, from
+    the restored prefix, gives the bits of one before."""
+    import torch
+    import paper_2609_37617_gb300 as lib
+    instr = torch_tokens(pair.cfg, n)
+    st = pair.state([L0], L0 + 512, [0])
+    first = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def prefill():
+        st.prefill(instr, first)
+        torch.cuda.synchronize()
+        got = (int(first.item()), bf16_bits(st.kc)[:, 0, :, :L0 + n], bf16_bits(st.vc)[:, 0, :, :L0 + n])
+        st.rollback([L0], [0])
+        return got
+
+    want = prefill()
+    st.check()
+    for limit in (0, 2000, 8000, 16000, 24000):
+        st.set_wait_limit(limit)
+        for _ in range(3):
+            prefill()
+        try:
+            st.check()
+            assert limit > 0, "a limit of 0 runs out"
+        except lib.AS2DError as e:
+            assert e.status == lib.AS2D_ERR_DEVICE and "timed out" in str(e)
+        st.set_wait_limit(2_000_000_000)
+        for a, b in zip(prefill(), want):
+            assert np.array_equal(a, b), limit
+        st.check()
+    st.close()
+
+
 def graph_node_types(graph):
     """cudaGraphNodeType of every node of a cudaGraph_t."""
     rt = ctypes.CDLL("libcudart.so.13")
