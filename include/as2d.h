@@ -176,7 +176,10 @@ as2d_status as2d_verify_block(as2d_kv* kv, const int32_t* candidates,
    also written to first_token (device int32 [1]) unless it is NULL.
    AS2D_ERR_UNSUPPORTED for batch > 1, AS2D_ERR_CAPACITY when the length
    bound plus n exceeds the capacity; bad token ids are device errors
-   (as2d_kv_check).  Asynchronous on `stream`. */
+   (as2d_kv_check): a pass that holds one keeps none of its rows, the other
+   passes' rows are kept, the root is the greedy token after the last row kept
+   (unchanged where there is none), and first_token is -1 if the last pass is
+   the one.  Asynchronous on `stream`. */
 as2d_status as2d_prefill(as2d_kv* kv, const int32_t* tokens, int32_t n,
                          int32_t* first_token, void* stream);
 

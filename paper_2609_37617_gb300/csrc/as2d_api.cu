@@ -561,10 +561,11 @@ cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, co
 // One verification pass.  mode: kAcceptVerify, or for a prefill's passes
 // (batch 1) every row kept and the LM head run over the pass's last row
 // (kAcceptAll) or not at all (kAcceptAllNoRoot); root_override: device int32
-// [batch], the tokens forwarded in place of the pending roots.
+// [batch], the tokens forwarded in place of the pending roots; keep: the
+// pass's part in a prefill of several.
 as2d_status run_block(KvState& s, const int32_t* cand, const int32_t* k,
                       const as2d_verify_out* out, cudaStream_t st, AcceptMode mode = kAcceptVerify,
-                      const int32_t* root_override = nullptr) {
+                      const int32_t* root_override = nullptr, KeepRow keep = kKeepNone) {
   if (!out || !out->n_accepted || !out->correction_token)
     return fail(AS2D_ERR_INVALID_ARG, "out, out->n_accepted and out->correction_token are required");
   RowMap rm;
@@ -615,11 +616,12 @@ as2d_status run_block(KvState& s, const int32_t* cand, const int32_t* k,
     tp.g_next = (l + 1 < c.n_layers) ? m.attn_norm[l + 1] : m.final_norm;
     LAUNCH(AS2D_KERNEL_DOWN, tc_project(TC_RESID, m, s, rm, m.w_down[l], m.tm_down[l], u, H, F, tp, st));
   }
+  if (keep != kKeepNone) LAUNCH(AS2D_KERNEL_OTHER, launch_keep_row(m, s, keep, rm.rows - 1, st));
   // a prefill needs one token, the greedy one after its last row
   if (mode != kAcceptAllNoRoot)
     LAUNCH(AS2D_KERNEL_LM_HEAD, tc_project(TC_LOGITS, m, s, rm, m.lm_head, m.tm_lm_head, xn, c.vocab, H, tp,
                                            st, mode == kAcceptAll ? rm.rows - 1 : 0));
-  LAUNCH(AS2D_KERNEL_OTHER, launch_accept(rm, m, s, cand, *out, st, mode));
+  LAUNCH(AS2D_KERNEL_OTHER, launch_accept(rm, m, s, cand, *out, st, mode, keep == kKeepRestore));
   for (int b = 0; b < s.batch; ++b) s.len_upper[b] += (k ? k[b] : 0) + 1;
   return AS2D_OK;
 }
@@ -679,6 +681,9 @@ as2d_status make_prefill_state(KvState& s, int rows) {
   a->d_root = s.d_root;
   a->d_err = s.d_err;
   a->rope_full = s.rope_full;
+  a->kept = s.kept;
+  a->kept_x = s.kept_x;
+  a->kept_ss = s.kept_ss;
   a->pf = s.pf;
   s.pf = a;
   return AS2D_OK;
@@ -695,11 +700,15 @@ as2d_status ensure_prefill_state(KvState& s, int want, cudaStream_t st) {
       cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
   const RelaxedCapture relaxed;
   if (!s.pf_out) {
-    const cudaError_t e = cudaMalloc(&s.pf_out, 2 * sizeof(int32_t));
+    const size_t H = s.model->cfg.hidden;
+    const cudaError_t e = cudaMalloc(&s.pf_out, 256 + 2 * H * sizeof(bf16) + H / 128 * sizeof(float));
     if (e != cudaSuccess) {
       s.pf_out = nullptr;
       return fail(AS2D_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     }
+    s.kept = s.pf_out + 2;
+    s.kept_x = (bf16*)((char*)s.pf_out + 256);
+    s.kept_ss = (float*)(s.kept_x + 2 * H);
   }
   const int least = prefill_rows(1);
   as2d_status rc = AS2D_OK;
@@ -748,8 +757,9 @@ extern "C" as2d_status as2d_prefill(as2d_kv* kh, const int32_t* tokens, int32_t 
     const bool last = s0 + rows == n;
     const as2d_verify_out out{s.pf_out, (last && first_token) ? first_token : s.pf_out + 1,
                               nullptr, nullptr};
+    const KeepRow keep = last ? (s0 > 0 ? kKeepRestore : kKeepNone) : s0 > 0 ? kKeepNext : kKeepFirst;
     rc = run_block(w, tokens + s0 + 1, &k, &out, (cudaStream_t)stream,
-                   last ? kAcceptAll : kAcceptAllNoRoot, /*root_override=*/tokens + s0);
+                   last ? kAcceptAll : kAcceptAllNoRoot, /*root_override=*/tokens + s0, keep);
   }
   s.len_upper = w.len_upper;
   s.launches += w.launches;

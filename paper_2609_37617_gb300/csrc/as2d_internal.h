@@ -29,6 +29,9 @@ inline int prefill_rows(int n) { return n <= 64 ? 64 : n <= 128 ? 128 : kPrefill
 // head).
 enum AcceptMode : int32_t { kAcceptVerify = 0, kAcceptAll = 1, kAcceptAllNoRoot = 2 };
 
+// What a pass of a prefill does with KvState::kept (k_basic.cu, keep_row_kernel).
+enum KeepRow : int32_t { kKeepNone = 0, kKeepFirst, kKeepNext, kKeepRestore };
+
 typedef __nv_bfloat16 bf16;
 
 // Row layout of one call: request b owns rows [start[b], start[b+1]); its
@@ -238,7 +241,12 @@ struct KvState {
   // candidates [batch][kMaxK], then n_accepted [batch] and correction [batch]
   int32_t* cb_dev = nullptr;
   int32_t* cb_host = nullptr;            // pinned, same layout
-  int32_t* pf_out = nullptr;             // [2] n_accepted, root of as2d_prefill chunks
+  int32_t* pf_out = nullptr;             // [2] n_accepted, root of as2d_prefill chunks; then kept, kept_x, kept_ss
+  // a prefill of several passes: whether one of them so far was kept, and the
+  // LM head's operand of the last row kept
+  int32_t* kept = nullptr;
+  bf16* kept_x = nullptr;                // [2][hidden] hi, lo
+  float* kept_ss = nullptr;              // [hidden / 128]
   // as2d_prefill's working state (batch 1, prefill_rows(n) rows per pass), made
   // on first use and a larger one for a longer call, the smaller behind it in
   // its own pf; shares this state's cache, lengths, roots, error flags and
@@ -257,7 +265,9 @@ cudaError_t launch_embed(const RowMap& m, const Model& md, KvState& kv,
                          const int32_t* root_override = nullptr);
 cudaError_t launch_accept(const RowMap& m, const Model& md, KvState& kv,
                           const int32_t* cand, const as2d_verify_out& out,
-                          cudaStream_t st, AcceptMode mode = kAcceptVerify);
+                          cudaStream_t st, AcceptMode mode = kAcceptVerify,
+                          bool kept_root = false);
+cudaError_t launch_keep_row(const Model& md, KvState& kv, KeepRow op, int row, cudaStream_t st);
 cudaError_t launch_rollback(KvState& kv, const int32_t* new_len,
                             const int32_t* new_root, cudaStream_t st);
 // Fills kv.rope_full for positions [0, capacity).

@@ -78,6 +78,34 @@ __global__ void accept_kernel(AcceptArgs a) {
   accept_request(a, blockIdx.x, threadIdx.x);
 }
 
+// A prefill of several passes runs the LM head over its last row alone.  If its
+// last pass is flagged, the root is the greedy token after the last row that
+// was kept: a pass before the last that is kept (kKeepFirst, kKeepNext) leaves
+// the LM head's operand of its last row, and a flagged last pass (kKeepRestore)
+// takes it up in the place of its own.
+__global__ void __launch_bounds__(256) keep_row_kernel(int32_t op, const int32_t* bad, int32_t* kept,
+                                                       bf16* xn, size_t lo, int H, float* ss, int ss_ld,
+                                                       bf16* kept_x, float* kept_ss) {
+  ptx::griddep_launch_dependents();
+  ptx::griddep_wait();
+  const bool flagged = *bad != 0, restore = op == kKeepRestore;
+  if (threadIdx.x == 0 && !restore && (op == kKeepFirst || !flagged)) *kept = flagged ? 0 : 1;
+  if (restore ? !(flagged && *kept) : flagged) return;
+  for (int c = threadIdx.x; c < H; c += 256) {
+    bf16 *x = xn + c, *k = kept_x + c;
+    if (restore)
+      x[0] = k[0], x[lo] = k[H];
+    else
+      k[0] = x[0], k[H] = x[lo];
+  }
+  for (int t = threadIdx.x; t < H / 128; t += 256) {
+    if (restore)
+      ss[(size_t)t * ss_ld] = kept_ss[t];
+    else
+      kept_ss[t] = ss[(size_t)t * ss_ld];
+  }
+}
+
 struct RollbackArgs {
   int32_t batch;
   int32_t len[kMaxBatch];
@@ -125,12 +153,20 @@ cudaError_t launch_rope_table(const Model& md, KvState& kv, cudaStream_t st) {
 
 cudaError_t launch_accept(const RowMap& m, const Model& md, KvState& kv,
                           const int32_t* cand, const as2d_verify_out& out,
-                          cudaStream_t st, AcceptMode mode) {
+                          cudaStream_t st, AcceptMode mode, bool kept_root) {
   (void)md;
   ++kv.launches;
   AcceptArgs a{m, cand, kv.best, kv.d_len, kv.d_root, kv.d_err + 1, out.n_accepted,
-               out.correction_token, out.greedy, mode};
+               out.correction_token, out.greedy, mode, kept_root ? kv.kept : nullptr};
   return launch_pdl(accept_kernel, dim3(m.batch), dim3(32), 0, st, 1, a);
+}
+
+cudaError_t launch_keep_row(const Model& md, KvState& kv, KeepRow op, int row, cudaStream_t st) {
+  ++kv.launches;
+  const int H = md.cfg.hidden;
+  return launch_pdl(keep_row_kernel, dim3(1), dim3(256), 0, st, 1, (int32_t)op,
+                    (const int32_t*)(kv.d_err + 1), kv.kept, kv.xn + (size_t)row * H,
+                    (size_t)kv.rows_alloc * H, H, kv.ss + row, kv.rows_alloc, kv.kept_x, kv.kept_ss);
 }
 
 cudaError_t launch_rollback(KvState& kv, const int32_t* new_len,

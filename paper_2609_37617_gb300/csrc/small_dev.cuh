@@ -75,6 +75,9 @@ struct AcceptArgs {
   int32_t* corr_out;
   int32_t* greedy_out;
   int32_t mode;  // AcceptMode
+  // kAcceptAll, nullable: whether an earlier pass of the prefill was kept (the
+  // greedy token of a flagged pass is then the one after the last row kept)
+  const int32_t* kept;
 };
 
 // Accept scan of request b by one warp (App. C.2): g_i from the packed maxima,
@@ -102,6 +105,7 @@ __device__ __forceinline__ void accept_request(const AcceptArgs& a, int b, int l
         a.n_out[b] = -1;
         a.corr_out[b] = -1;
         a.bad[b] = 0;
+        if (a.kept && *a.kept) a.root[b] = g_last;
       } else {
         a.n_out[b] = k;
         a.len[b] += k + 1;

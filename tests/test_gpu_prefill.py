@@ -203,6 +203,37 @@ def test_first_prefill_under_capture(pair, mode):
     ref.close()
 
 
+# passes of 150 + 150 and of 256 + 256 + 88 rows
+@pytest.mark.parametrize("n,bad,kept", [(300, [299], [(0, 150)]), (300, [0], [(150, 300)]), (300, [3, 200], []),
+                                        (600, [512], [(0, 512)]), (600, [256, 520], [(0, 256)]),
+                                        (600, [255, 599], [(256, 512)]), (600, [10, 500], [(512, 600)])])
+def test_prefill_root_after_flagged_pass(pair, n, bad, kept):
+    """Bad token ids flag their passes: the state is the one after the rows of
+    the other passes alone, its root the greedy token after the last of them."""
+    import torch
+    import paper_2609_37617_gb300 as lib
+    instr = torch_tokens(pair.cfg, n)
+    broken = instr.clone()
+    broken[bad] = torch.tensor([pair.cfg.vocab, -1][:len(bad)], dtype=torch.int32, device="cuda")
+    first = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref = pair.state([L0], L0 + 700, [7])
+    for a, b in kept:
+        ref.prefill(instr[a:b], first)
+    for warm in (False, True):  # the second time after a call that kept every pass
+        st = pair.state([L0], L0 + 700, [7])
+        if warm:
+            st.prefill(instr, first)
+            st.rollback([L0], [7])
+        st.prefill(broken, first)
+        torch.cuda.synchronize()
+        with pytest.raises(lib.AS2DError):
+            st.check()
+        assert st.read_state() == ref.read_state()
+        assert (int(first.item()) == -1) == (max(bad) >= {300: 150, 600: 512}[n])
+        st.close()
+    ref.close()
+
+
 @pytest.mark.parametrize("n", [40, 100, 300])
 def test_prefill_recovers_from_expired_waits(pair, n):
     """A prefill whose kernels' waits run out reports it; the next one, from
