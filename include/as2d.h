@@ -121,7 +121,11 @@ as2d_status as2d_model_load(const as2d_config* cfg, const as2d_weights* w,
 /* Size this model's kernel grids for n_sms SMs (1 .. the device's count; the
    default is the device's count), so that the pass can share the GPU with
    other work confined to the remaining SMs -- for example a drafter on its
-   own stream (as2d_session_run).  The work split depends on (shape, n_sms)
+   own stream (as2d_session_run).  The projections' grids are of CTAs in
+   groups of two, one CTA to an SM: an odd n_sms leaves one SM unused, 1 counts
+   as 2, and the QKV projection, which has a CTA or more to each 128 of its
+   rows, may start CTAs beyond n_sms that take the SMs in turn.  The other
+   kernels are not sized.  The work split depends on (shape, n_sms)
    only: results stay batch invariant and bit-identical for a given budget;
    another budget adds partial sums in another order.  States created before
    a larger budget was set refuse to run (AS2D_ERR_INVALID_ARG): set the

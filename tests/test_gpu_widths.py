@@ -35,8 +35,9 @@ def test_rows(pair, rows):
 
 # Few SMs give each CTA enough units for pairs of CTAs: with 2, whole tiles of
 # odd counts (gate/up 23, down 3, vocabulary 9), with 4 also tiles of the
-# residual projections cut between CTAs.  NB = 64, 96, 192, 256 and 16.
-@pytest.mark.parametrize("sms", [2, 4])
+# residual projections cut between CTAs.  NB = 64, 96, 192, 256 and 16.  (A
+# budget of 1 runs as 2, one of 3 on the groups of 2.)
+@pytest.mark.parametrize("sms", [1, 2, 3, 4])
 @pytest.mark.parametrize("rows", [[16] * 4, [17] * 4, [17] * 10, [17] * 16], ids=lambda r: f"{sum(r)}rows")
 def test_rows_few_sms(rows, sms):
     import torch
