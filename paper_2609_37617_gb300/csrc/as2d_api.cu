@@ -479,17 +479,18 @@ struct Operand {
   const CUtensorMap *maps, *pair;  // per token-row padding
 };
 
-// Rows of a projection's next launch, of `left`: equal shares where they pad
-// to 160 or 192 rows, else 256 first.  Whole passes, us, 256 first against
+// Rows of a projection's launches, of `left` left: equal shares (the result)
+// where these pad to 160 rows, or to 192 and to no more in total than 256 first
+// (from 353 rows); else 0, 256 first.  Whole passes, us, 256 first against
 // shares: 272 / 306 / 320 / 384 rows of the 1.5B 3324 / 3509 / 3594 / 3909
 // against 3298 / 3434 / 3517 / 3798, of the 7B 8467 / 8700 / 8840 / 9713
-// against 8245 / 8440 / 8560 / 9580; 576 rows as 3 x 192 against 256 + 160 +
-// 160 6404 / 6572 and 14460 / 14945; 256 + 96 is the better of 2 x 176 (352
-// rows 3700 / 3709 and 9370 / 9470), and 256 + 134 of 2 x 195.
-int launch_rows(int left) {
+// against 8245 / 8440 / 8560 / 9580; 513 / 529 / 576 rows in two launches after
+// 256 against three shares 5511 / 5629 / 6572 against 5443 / 5486 / 6404 and
+// 13909 / 14479 / 14945 against 13994 / 14158 / 14460; 256 + 96 is the better of
+// 2 x 176 (352 rows 3700 / 3709 and 9370 / 9470), and 256 + 134 of 2 x 195.
+int equal_share(int left) {
   const int n = (left + 255) / 256, share = (left + n - 1) / n;
-  if (n == 1) return left;
-  return share <= 160 || (share <= 192 && left > 352) ? share : 256;
+  return n == 1 || share <= 160 || (share <= 192 && left > 352) ? share : 0;
 }
 
 cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, const bf16* w,
@@ -540,9 +541,12 @@ cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, co
   p.err = s.d_err;
   p.timeout_ns = s.wait_ns;
   p.rm = rm;
-  for (int row0 = first_row; row0 < rm.rows; row0 += p.rows) {
+  // (shares once taken stand for the launches that follow)
+  for (int row0 = first_row, share = 0; row0 < rm.rows; row0 += p.rows) {
+    const int left = rm.rows - row0;
+    if (share == 0) share = equal_share(left);
     p.row0 = row0;
-    p.rows = launch_rows(rm.rows - row0);
+    p.rows = share == 0 ? 256 : left < share ? left : share;
     const int nb = nb_for_rows(p.rows), i = nb_index(nb);
     const TcMaps maps{&x.maps[i], &x.pair[i], &wmap};
     cudaError_t e;

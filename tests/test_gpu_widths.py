@@ -24,10 +24,11 @@ def pair():
 
 # requests x rows: 1, 15, 16, 17 (a finishing CTA's rows), then one call past
 # each padding's lower edge and at 256, 257, 272 and 320 rows (two halves), 323 (256
-# and the rest), 353 (two), 391 (256 and the rest), 544 (three)
+# and the rest), 353 (two), 391 (256 and the rest), 513, 529 and 544 (three)
 @pytest.mark.parametrize("rows", [[1], [15], [16], [17], [17, 16], [17, 17, 15], [16] * 4, [17] * 4, [17] * 6,
                                   [17] * 8, [17] * 10, [17] * 12, [16] * 16, [17] * 15 + [2], [17] * 16,
-                                  [17] * 18 + [14], [17] * 19, [17] * 20 + [13], [17] * 23, [17] * 32],
+                                  [17] * 18 + [14], [17] * 19, [17] * 20 + [13], [17] * 23, [17] * 30 + [3],
+                                  [17] * 31 + [2], [17] * 32],
                          ids=lambda r: f"{sum(r)}rows")
 def test_rows(pair, rows):
     check_rows(pair, rows)
