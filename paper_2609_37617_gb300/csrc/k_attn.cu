@@ -61,6 +61,7 @@
 // not depend on the other rows of the call (batch invariance).
 #include "as2d_internal.h"
 #include "ptx_sm100.cuh"
+#include "quotient.cuh"
 
 namespace as2d {
 namespace {
@@ -380,9 +381,8 @@ __device__ __forceinline__ void softmax_tail(float (&sv)[32], int c, int p0, int
 
 // Positions [fd, fd + DT) (fd a multiple of DT) of row fr of query tile qt,
 // normalised (o / l), as bf16 hi and lo parts into the attention output; rows
-// past the call's queries are skipped.  The quotients are x r, r = 1 / l, with
-// one correction by their remainder (Markstein's method: within a rounding of
-// the quotient), as eight divisions in a row would hold up the chain.
+// past the call's queries are skipped.  One reciprocal serves the row
+// (quotient.cuh), as eight divisions in a row would hold up the chain.
 template <int D, int DT>
 __device__ __forceinline__ void write_rows(const AttnArgs& a, const float* o_, float Ls, int fr,
                                            int fd, int qt, int qn, int G, int g, int r0) {
@@ -396,10 +396,7 @@ __device__ __forceinline__ void write_rows(const AttnArgs& a, const float* o_, f
   for (int e = 0; e < DT / 2; ++e) {
     float v[2];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const float x = o_[2 * e + u] * inv;
-      v[u] = fmaf(fmaf(-x, Ls, o_[2 * e + u]), inv, x);
-    }
+    for (int u = 0; u < 2; ++u) v[u] = quotient(o_[2 * e + u], Ls, inv);
     const __nv_bfloat162 hv = __floats2bfloat162_rn(v[0], v[1]);
     const float2 hf = __bfloat1622float2(hv);
     const __nv_bfloat162 lv = __floats2bfloat162_rn(v[0] - hf.x, v[1] - hf.y);
