@@ -540,7 +540,6 @@ cudaError_t tc_project(int epi, const Model& m, KvState& s, const RowMap& rm, co
   p.counters = s.counters;
   p.err = s.d_err;
   p.timeout_ns = s.wait_ns;
-  p.rm = rm;
   // (shares once taken stand for the launches that follow)
   for (int row0 = first_row, share = 0; row0 < rm.rows; row0 += p.rows) {
     const int left = rm.rows - row0;

@@ -109,7 +109,6 @@ struct TcParams {
   int n_htiles;          // hidden / 128 (consumer side)
   float eps;
   int hidden;
-  RowMap rm;
 };
 
 // Launch with programmatic stream serialization: the kernel may be scheduled

@@ -84,7 +84,7 @@ static_assert(kStage * 8 * 128 * 4 + kStage * 8 * 8 <= 2 * 32768, "staging fits 
 // memory.
 template <bool NARROW, bool PAIR>
 constexpr uint32_t attn_smem() {
-  return (NARROW ? 2 : 3) * 32768 + 64 * 8 + 8 * 4 + 5 * 8 + 16 + 1024;
+  return (NARROW ? 2 : 3) * 32768 + 64 * 8 + 5 * 8 + 16 + 1024;
 }
 static_assert(3 * (attn_smem<true, false>() + 1024) <= 228 * 1024, "three narrow CTAs per SM");
 static_assert(2 * (attn_smem<false, true>() + 1024) <= 228 * 1024, "two wide CTAs per SM");
@@ -459,14 +459,13 @@ __device__ __forceinline__ void fold_tiles(const float* o, int stride, const flo
 // what follows it: with one chunk the rows are normalised and written; with
 // several, the rows of the chunk partial go to memory, for attn_fold_kernel
 // (fold_later) or for the last CTA of these rows to arrive, which folds the
-// chunks in chunk order (9 to stage_max chunks staged in shared memory at sm,
-// whose images are no longer read).
-template <int D>
+// chunks in chunk order (9 to STAGE chunks staged in shared memory at sm,
+// whose images are no longer read; none with STAGE 0).
+template <int D, int STAGE>
 __device__ __forceinline__ void fold_chunk8(const AttnArgs& a, const float* recv,
                                             const float2* s_rml, int* s_flag, uint8_t* sm,
-                                            int stage_max, uint32_t rank, int c, int n_tiles,
-                                            int n_chunks, int b, int g, int qt, int qn, int G,
-                                            int r0) {
+                                            uint32_t rank, int c, int n_tiles, int n_chunks, int b,
+                                            int g, int qt, int qn, int G, int r0) {
   constexpr int DT = D / 16;  // dims per thread (8 rows x 16 threads)
   const int tid = threadIdx.x;
   // ---- fold (thread: query row 8 rank + fj, positions [fd, fd + DT)) ----------
@@ -516,43 +515,45 @@ __device__ __forceinline__ void fold_chunk8(const AttnArgs& a, const float* recv
   float cl_ = 0.f, co[DT];
 #pragma unroll
   for (int e = 0; e < DT; ++e) co[e] = 0.f;
-  if (n_chunks > 8 && n_chunks <= stage_max) {
-    // nine or more chunks: every chunk's rows come into shared memory (over
-    // the Q / P and K images, no longer read) by copies issued together, one
-    // memory round trip instead of two through registers
-    float* st_o = reinterpret_cast<float*>(sm);                          // [chunk][8 rows][D]
-    float2* st_ml = reinterpret_cast<float2*>(sm + stage_max * 8 * D * 4);  // [chunk][8 rows]
-    for (int cc = 0; cc < n_chunks; ++cc) {
-      const size_t pc = item * a.chunks_max + cc;
-      const float* src = a.ws_o + (pc * kQT + fr) * D + fd;
-      float* dst = st_o + (cc * 8 + fj) * D + fd;
-#pragma unroll
-      for (int u = 0; u < DT / 4; ++u) ptx::cp_async16(dst + 4 * u, src + 4 * u);
-      // (max, sum) of rows fj and fj + 1 in one copy
-      if ((tid & 15) == 0 && (fj & 1) == 0) ptx::cp_async16(st_ml + cc * 8 + fj, a.ws_ml + pc * kQT + fr);
-    }
-    ptx::cp_async_wait_all();
-    __syncthreads();
-    float cm = -INFINITY;
-    for (int cc = 0; cc < n_chunks; ++cc) cm = fmaxf(cm, st_ml[cc * 8 + fj].x);
-    for (int cc = 0; cc < n_chunks; ++cc) {
-      const float2 ml = st_ml[cc * 8 + fj];
-      const float w = part_weight(ml.x, cm);
-      if (w != 0.f) {
-        cl_ += ml.y * w;
-        const float4* src = reinterpret_cast<const float4*>(st_o + (cc * 8 + fj) * D + fd);
-#pragma unroll
-        for (int u = 0; u < DT / 4; ++u) {
-          const float4 v = src[u];
-          co[4 * u + 0] += v.x * w;
-          co[4 * u + 1] += v.y * w;
-          co[4 * u + 2] += v.z * w;
-          co[4 * u + 3] += v.w * w;
+  if constexpr (STAGE > 0) {
+    if (n_chunks > 8 && n_chunks <= STAGE) {
+      // nine or more chunks: every chunk's rows come into shared memory (over
+      // the Q / P and K images, no longer read) by copies issued together, one
+      // memory round trip instead of two through registers
+      float* st_o = reinterpret_cast<float*>(sm);                          // [chunk][8 rows][D]
+      float2* st_ml = reinterpret_cast<float2*>(sm + STAGE * 8 * D * 4);  // [chunk][8 rows]
+      for (int cc = 0; cc < n_chunks; ++cc) {
+        const size_t pc = item * a.chunks_max + cc;
+        const float* src = a.ws_o + (pc * kQT + fr) * D + fd;
+        float* dst = st_o + (cc * 8 + fj) * D + fd;
+  #pragma unroll
+        for (int u = 0; u < DT / 4; ++u) ptx::cp_async16(dst + 4 * u, src + 4 * u);
+        // (max, sum) of rows fj and fj + 1 in one copy
+        if ((tid & 15) == 0 && (fj & 1) == 0) ptx::cp_async16(st_ml + cc * 8 + fj, a.ws_ml + pc * kQT + fr);
+      }
+      ptx::cp_async_wait_all();
+      __syncthreads();
+      float cm = -INFINITY;
+      for (int cc = 0; cc < n_chunks; ++cc) cm = fmaxf(cm, st_ml[cc * 8 + fj].x);
+      for (int cc = 0; cc < n_chunks; ++cc) {
+        const float2 ml = st_ml[cc * 8 + fj];
+        const float w = part_weight(ml.x, cm);
+        if (w != 0.f) {
+          cl_ += ml.y * w;
+          const float4* src = reinterpret_cast<const float4*>(st_o + (cc * 8 + fj) * D + fd);
+  #pragma unroll
+          for (int u = 0; u < DT / 4; ++u) {
+            const float4 v = src[u];
+            co[4 * u + 0] += v.x * w;
+            co[4 * u + 1] += v.y * w;
+            co[4 * u + 2] += v.z * w;
+            co[4 * u + 3] += v.w * w;
+          }
         }
       }
+      write_out(co, cl_);
+      return;
     }
-    write_out(co, cl_);
-    return;
   }
   // eight chunks' values in flight at a time; the first eight are requested
   // together with every chunk's maximum, so that up to eight chunks take one
@@ -573,9 +574,9 @@ __device__ __forceinline__ void fold_chunk8(const AttnArgs& a, const float* recv
   // more chunks than shared memory holds, but no more than eight plus that:
   // chunks 8.. come into shared memory by copies issued together with the
   // first eight's loads, so that all of them take one memory round trip
-  const bool hybrid = n_chunks > 8 && n_chunks - 8 <= stage_max;
+  const bool hybrid = STAGE > 0 && n_chunks > 8 && n_chunks - 8 <= STAGE;
   float* st_o = reinterpret_cast<float*>(sm);                          // [chunk - 8][8 rows][D]
-  float2* st_ml = reinterpret_cast<float2*>(sm + stage_max * 8 * D * 4);  // [chunk - 8][8 rows]
+  float2* st_ml = reinterpret_cast<float2*>(sm + STAGE * 8 * D * 4);  // [chunk - 8][8 rows]
   if (hybrid) {
     for (int cc = 8; cc < n_chunks; ++cc) {
       const size_t pc = item * a.chunks_max + cc;
@@ -654,8 +655,7 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
   float* recv = reinterpret_cast<float*>(R1);  // [8 tiles][8 rows][D] received
   // [tiles of the cluster][rows folded here] (max, sum): [8][8], pair [16][4]
   float2* s_rml = reinterpret_cast<float2*>(sm + (NARROW ? 2 : 3) * 32768);
-  float* s_x = reinterpret_cast<float*>(s_rml + 64);      // [8] scratch
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_x + 8);  // q, k (wide: and v), mma1, mma2, v
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_rml + 64);  // q, k (wide: and v), mma1, mma2, v
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 5);
   int* s_flag = reinterpret_cast<int*>(tslot + 1);
 
@@ -947,8 +947,7 @@ __global__ void __launch_bounds__(128, NARROW ? 3 : 2)
     return;
   }
 
-  fold_chunk8<D>(a, recv, s_rml, s_flag, sm, kStage, rank, c, n_tiles, n_chunks, b, g, qt, qn, G,
-                 r0);
+  fold_chunk8<D, kStage>(a, recv, s_rml, s_flag, sm, rank, c, n_tiles, n_chunks, b, g, qt, qn, G, r0);
 }
 
 // Four CTAs per SM (QUAD), for launches of more clusters than the narrow
@@ -1175,7 +1174,7 @@ __global__ void __launch_bounds__(128, 4)
     }
   }
   ptx::cluster_sync();
-  fold_chunk8<D>(a, recv, s_rml, s_flag, sm, 0, rank, c, n_tiles, n_chunks, b, g, qt, qn, G, r0);
+  fold_chunk8<D, 0>(a, recv, s_rml, s_flag, sm, rank, c, n_tiles, n_chunks, b, g, qt, qn, G, r0);
 }
 
 // The chunk partials of attn_tc4_kernel's requests of several chunks, folded in
