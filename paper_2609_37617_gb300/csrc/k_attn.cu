@@ -50,11 +50,9 @@
 // per SM in 48 KB, for launches of more clusters than the narrow layout
 // keeps resident.
 // Bound by latency: each CTA is one dependent chain, of which an SM overlaps
-// two to four.  With hi and lo rows in adjacent lanes, exchanged by shuffles, a
-// tile spent 2.4 us of its chain on instructions (read S 0.4, softmax 0.5, write
-// P 0.7, read O 0.75, measured); with both parts in one thread 1.5B k = 0 takes
-// 1111 -> 1079 us a pass, 7B k = 8 2749 -> 2692, L = 15128 k = 16 3616 -> 3388, 16
-// ragged requests 7014 -> 6384.
+// two to four.  With both parts of a query in one thread a pass takes 1079 us
+// (1.5B, k = 0) and 2692 (7B, k = 8), with the parts in adjacent lanes,
+// exchanged by shuffles, 1111 and 2749.
 // Every fold boundary is a fixed absolute key position (128-key tiles,
 // 1024-key chunks), and a fold with a part a row cannot see (fully masked:
 // m = -inf, l = 0, O = 0) leaves it bitwise unchanged, so a row's result does
@@ -89,12 +87,15 @@ constexpr uint32_t attn_smem() {
 static_assert(3 * (attn_smem<true, false>() + 1024) <= 228 * 1024, "three narrow CTAs per SM");
 static_assert(2 * (attn_smem<false, true>() + 1024) <= 228 * 1024, "two wide CTAs per SM");
 // A launch of more clusters of 8 than this takes the narrow layout.  The wide
-// kernel's shared memory allows 36 clusters of 8 at two CTAs per SM (the
-// occupancy calculator reports 15); measured on 7B and 1.5B calls, the wide
-// layout is the faster up to 32 clusters and much the slower at 36.
+// kernel's shared memory allows 36 clusters of 8 at two CTAs per SM.  Passes,
+// us, wide / narrow: 7B, k = 8 with 32 clusters 2834 / 2860, 36 2847 / 2872,
+// 40 3009 / 2880; blocks of the 1.5B with 32 1420 / 1464, 36 1472 / 1500, 40
+// 1663 / 1520.
 constexpr int kWideClusters = 32;
-// clusters of 8 the narrow layout keeps resident (three CTAs per SM, residency
-// probe); larger launches take four CTAs per SM
+// Clusters of 8 the narrow layout keeps resident (three CTAs per SM, residency
+// probe); larger launches take four CTAs per SM.  Passes, us, narrow / four:
+// 7B, k = 8 with 48 clusters 2918 / 2938, 52 3029 / 2949, 60 3081 / 2978; blocks
+// of the 1.5B with 48 1624 / 1638, 52 1772 / 1685.
 constexpr int kNarrowClusters = 51;
 
 struct AttnArgs {
@@ -422,9 +423,8 @@ __device__ __forceinline__ void write_rows(const AttnArgs& a, const float* o_, f
 // maxima m, -inf for none): o and l relative to the largest, fm.  Every load is
 // issued before the first is used, and parts of weight 0 are dropped by
 // selection (what lies in their place is not read into the sums).  The fold
-// stands at the end of every layer's chain: 1.5 us with a branch for each part
-// and eight divisions; without them 1.5B k = 0 / 8 1069 -> 1058 / 1142 -> 1115 us
-// a pass, 7B k = 8 2699 -> 2689, L = 15128 k = 16 3385 -> 3352.
+// stands at the end of every layer's chain: with a branch for each part and
+// eight divisions it took 1.5 us (1.5B, k = 8 1142 us a pass, now 1115).
 template <int NT, int DT>
 __device__ __forceinline__ void fold_tiles(const float* o, int stride, const float2 (&ml)[NT], float& fm,
                                            float& fl, float (&fo)[DT]) {
@@ -1378,9 +1378,9 @@ cudaError_t launch_attention_split(const RowMap& m, const Model& md, KvState& kv
   // at most two chunks, and the clusters of 16 run at once.
   const bool narrow = clusters8 * c.n_kv_heads > kWideClusters;
   const bool quad = clusters8 * c.n_kv_heads > kNarrowClusters;
-  // Measured: the prefetch of V takes 32 µs off a 7B block at L = 15128 (60
-  // clusters of 8) and 12 µs at k = 16 (120), but adds 100 µs to a ragged
-  // round of 16 requests (about 440 clusters, some nine waves).
+  // Passes, us, without / with the prefetch of V: 36 clusters of 8 on the 7B
+  // 2877 / 2872, on the 1.5B 1509 / 1500; 60 (7B) 2972 / 2978; 128 3392 / 3400;
+  // 144 3447 / 3460; 16 ragged requests (about 440) 6127 / 6180.
   a.v_prefetch = clusters8 * c.n_kv_heads <= 128;
   int clusters16 = 0;
   for (int b = 0; b < kv.batch; ++b)

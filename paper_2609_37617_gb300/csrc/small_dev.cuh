@@ -23,9 +23,10 @@ __device__ __forceinline__ void embed_row_body(const bf16* __restrict__ e,
                                                bf16* __restrict__ xn, float* __restrict__ ss,
                                                int tid, int nthr, float* red, int bar_id) {
   // Bound by the latency of the table row's load from HBM: up to kBatch columns
-  // a thread are requested before the first is used.  As a plain loop, four;
-  // with the accept scan's loads together too, whole calls at k = 8 1125 ->
-  // 1116 us (1.5B), 2661 -> 2658 us (7B).
+  // a thread are requested before the first is used, so that the 12 of the 1.5B
+  // take one memory round trip and the 28 of the 7B two.  With 7 / 14 / 28 a
+  // pass takes 1075 / 1069 / 1072 us (1.5B, k = 0), 1110 / 1108 / 1111 (k = 8),
+  // 2613 / 2610 / 2608 (7B, k = 0), 2680 / 2681 / 2689 (k = 8).
   constexpr int kBatch = 14;
   float sq = 0.f;
   for (int c0 = tid; c0 < H; c0 += kBatch * nthr) {
