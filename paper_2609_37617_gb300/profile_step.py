@@ -10,7 +10,8 @@ uniform tokens, since a block's work does not depend on what is accepted.
 Each block starts from the same prefix (a rollback), so every captured launch
 sees the same length.  The blocks after the warm-up run inside the NVTX range
 "blocks" (ncu --nvtx --nvtx-include blocks/); each is a rollback launch and
-one verification pass of 3 + 9 x n_layers launches.
+one verification pass of 3 + 8 x n_layers launches (9 where chunk partials of
+long prefixes are folded by a kernel of their own; more above 256 token rows).
 """
 import argparse
 import os
