@@ -67,7 +67,7 @@ enum : int32_t {
 // Whether a request of device-side length `len` has room for `rows` more
 // cache entries.  A request that does not is skipped by every kernel that
 // indexes the cache or the rotary table with its length (no key/value append,
-// no attention, zero attention output); the embedding kernel flags it
+// no attention: its rows' results are undefined); the embedding kernel flags it
 // (kErrCapacity and the request's bad flag), and the accept scan then reports
 // n_accepted = correction = -1 and leaves its length and root unchanged.
 __host__ __device__ inline bool rows_fit(int len, int rows, int cap) {
