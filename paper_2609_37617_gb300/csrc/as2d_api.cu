@@ -643,12 +643,13 @@ struct RelaxedCapture {
   }
 };
 
-// Zeroes fresh device memory before it returns, on a stream of its own: on the
-// caller's the memset of a call under capture would only become a node of the
-// graph, and calls that run before that graph does (or without it, if it is
-// dropped) would find what the allocation held.
-cudaError_t zero_now(void* p, size_t bytes) {
-  cudaStream_t st = nullptr;
+// Zeroes fresh device memory: in the order of the caller's stream or, if that is
+// under capture, before it returns, on a stream of its own: on the caller's
+// the memset would only become a node of the graph, and calls that run before
+// that graph does (or without it, if it is dropped) would find what the
+// allocation held.
+cudaError_t zero_new(void* p, size_t bytes, cudaStream_t st, bool captured) {
+  if (!captured) return cudaMemsetAsync(p, 0, bytes, st);
   cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(p, 0, bytes, st);
@@ -660,7 +661,7 @@ cudaError_t zero_now(void* p, size_t bytes) {
 // A prefill working state of `rows` rows a pass, put before the ones that s
 // has: those stay until as2d_kv_free, as a captured graph may hold their
 // addresses (at most one of each of 64, 128 and 256 rows).
-as2d_status make_prefill_state(KvState& s, int rows) {
+as2d_status make_prefill_state(KvState& s, int rows, cudaStream_t st, bool captured) {
   KvState* a = new KvState();
   a->model = s.model;
   a->batch = 1;
@@ -670,7 +671,7 @@ as2d_status make_prefill_state(KvState& s, int rows) {
   a->len_upper = s.len_upper;
   as2d_status rc = alloc_work(*a, *s.model, 1, s.capacity, rows);
   if (rc == AS2D_OK) {
-    const cudaError_t e = zero_now(a->work, a->work_bytes);
+    const cudaError_t e = zero_new(a->work, a->work_bytes, st, captured);
     if (e != cudaSuccess) {
       cudaFree(a->work);
       rc = fail(AS2D_ERR_CUDA, std::string("zeroing the working memory: ") + cudaGetErrorString(e));
@@ -715,11 +716,8 @@ as2d_status ensure_prefill_state(KvState& s, int want, cudaStream_t st) {
   }
   const int least = prefill_rows(1);
   as2d_status rc = AS2D_OK;
-  if (!s.pf && captured)
-    rc = make_prefill_state(s, least);
-  else if (!captured && (!s.pf || want > s.pf->max_rows))
-    rc = make_prefill_state(s, want);
-  if (rc != AS2D_OK && !s.pf && !captured && want > least) rc = make_prefill_state(s, least);
+  if (!captured && (!s.pf || want > s.pf->max_rows)) rc = make_prefill_state(s, want, st, false);
+  if (!s.pf && (captured || want > least)) rc = make_prefill_state(s, least, st, captured);
   (void)cudaGetLastError();
   if (!s.pf) return rc;
   g_err.clear();
